@@ -270,21 +270,22 @@ QS_HD void two_sum2(float2 a, float2 b, float2& s, float2& e) {
   const float2 bb = sub2(s, a);
   e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
-// lane-wise TwoSum of a and -b: s + e == a - b exactly
-QS_HD void two_diff2(float2 a, float2 b, float2& s, float2& e) {
-  s = sub2(a, b);
-  const float2 bb = sub2(s, a);
-  e = sub2(sub2(a, sub2(s, bb)), add2(b, bb));
+// sign flip of both lanes (integer operations, not the FMA pipe)
+QS_HD float2 neg2(float2 a) {
+  return make_float2(f_from_bits(f_bits(a.x) ^ 0x80000000u), f_from_bits(f_bits(a.y) ^ 0x80000000u));
 }
-// Lane-wise double-float product of U = Uh + Ul (given as Uh, -Uh, -Ul) and v = vh + vl:
-// p = Uh vh rounded, ne = -(TwoProduct error + Uh vl + Ul vh), so that U v ~= p - ne
-// (the product of the low parts, ~2^-48 relative, is dropped).  The negated operands keep
-// every step a plain packed FMA: FMA(-Uh, vh, p) is the exact negated TwoProduct error.
-QS_HD void prod2(float2 Uh, float2 nUh, float2 nUl, float2 vh, float2 vl, float2& p, float2& ne) {
-  p = mul2(Uh, vh);
-  ne = fma2(nUh, vh, p);
-  ne = fma2(nUh, vl, ne);
-  ne = fma2(nUl, vh, ne);
+// Lane-wise s + d + c = a + U v to about 2^-48 |s|: TwoSum of a and p = RN(U v) in which the
+// FMA d = U v - (what p added to s) replaces TwoSum's last difference and the product's own
+// rounding error: 6 instructions where TwoProduct and TwoSum take 8.  s is the sum of two
+// floats and not one FMA of the exact product: under cancellation the FMA's result has bits
+// below ulp(a), and the differences with a would no longer be exact (errors of 2^-25).  The
+// product is therefore an FMA with 0: the assembler contracts a packed multiply whose only
+// use is a packed add, explicit .rn or not, and it leaves an FMA alone.
+QS_HD void add_prod2(float2 a, float2 U, float2 v, float2& s, float2& d, float2& c) {
+  s = add2(a, fma2(U, v, make_float2(0.f, 0.f)));
+  const float2 nb = sub2(a, s);       // -(what the product added)
+  d = fma2(U, v, nb);
+  c = sub2(a, add2(s, nb));
 }
 
 // Split a binary64 value into hi + lo floats without FP64 instructions.
@@ -350,10 +351,14 @@ QS_HD double join_double(float hi, float lo) {
 //
 // mat_t (48 bytes, prepared on the host) holds a complex u = ur + i ui as lane patterns:
 //   a = ( ur.hi,  ur.hi, -ur.hi, -ur.hi)     ur on both lanes, and its negation
-//   b = (-ui.hi,  ui.hi,  ui.hi, -ui.hi)     (-ui, ui): i ui acting on a swapped (im, re)
-//   c = (-ur.lo, -ur.lo,  ui.lo, -ui.lo)     negated low parts of both patterns
+//   b = (-ui.hi,  ui.hi,  ur.lo,  ur.lo)     (-ui, ui): i ui acting on a swapped (im, re); low part of ur
+//   c = (-ui.lo,  ui.lo, -ur.lo, -ur.lo)     low part of (-ui, ui); negated low part of ur
 // so that u a = ur (.) a + (-ui, ui) (.) swap(a) lane-wise and no packed operand needs a
-// sign flip at run time.
+// sign flip at run time (a real factor t = ur takes both signs from a, b and c).
+//
+// Instruction counts per amplitude (packed, two lanes each): u + t v 10, a complex product 14,
+// acc + u a 20.  Each sum of a value and a product is one add_prod2; with a TwoProduct and a
+// TwoSum the three took 12, 16 and 24.
 //
 // Tile passes run in a phase frame: amplitude i of a tile is held as (-i)^popcount(i)
 // times its value (S^dagger on every tile bit).  Diagonal gates are unchanged, RX becomes
@@ -364,10 +369,10 @@ QS_HD double join_double(float hi, float lo) {
 struct alignas(16) dfm {
   float4 a, b, c;
 };
-// a real double-float factor t as the three lane pairs the products need: (t.hi, t.hi),
-// its negation, and the negated low part
+// a real double-float factor t as the lane pairs the products need: high and low part on both
+// lanes, and their negations
 struct dfr {
-  float2 h, nh, nl;
+  float2 h, nh, l, nl;
 };
 
 struct ADF {
@@ -398,20 +403,30 @@ struct ADF {
     return *p;
 #endif
   }
-  // the real part of an entry (t, 0): two of its three 16-byte words
+  // the real part of an entry (t, 0)
   static QS_HD dfr ld_real(const mat_t* p) {
 #ifdef __CUDA_ARCH__
-    float4 a, c;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w) : "l"(p));
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4+32];" : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w) : "l"(p));
-    return dfr{make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(c.x, c.y)};
+    dfr r;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(r.h.x), "=f"(r.h.y), "=f"(r.nh.x), "=f"(r.nh.y) : "l"(p));
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+24];" : "=f"(r.l.x), "=f"(r.l.y) : "l"(p));
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+40];" : "=f"(r.nl.x), "=f"(r.nl.y) : "l"(p));
+    return r;
 #else
     return real_of(*p);
 #endif
   }
   static QS_HD dfr real_of(const mat_t& m) {
-    return dfr{make_float2(m.a.x, m.a.y), make_float2(m.a.z, m.a.w), make_float2(m.c.x, m.c.y)};
+    return dfr{make_float2(m.a.x, m.a.y), make_float2(m.a.z, m.a.w), make_float2(m.b.z, m.b.w),
+               make_float2(m.c.z, m.c.w)};
   }
+  // the lane patterns of an entry
+  static QS_HD float2 mA(const mat_t& m) { return make_float2(m.a.x, m.a.y); }     // ( ur,  ur)
+  static QS_HD float2 mnA(const mat_t& m) { return make_float2(m.a.z, m.a.w); }    // (-ur, -ur)
+  static QS_HD float2 mB(const mat_t& m) { return make_float2(m.b.x, m.b.y); }     // (-ui,  ui)
+  static QS_HD float2 mAl(const mat_t& m) { return make_float2(m.b.z, m.b.w); }    // low parts
+  static QS_HD float2 mnAl(const mat_t& m) { return make_float2(m.c.z, m.c.w); }
+  static QS_HD float2 mBl(const mat_t& m) { return make_float2(m.c.x, m.c.y); }
   static QS_HD reg_t from_store(store_t v) {
     const dfl r = split_double(v.x), i = split_double(v.y);
     return make_float4(r.hi, i.hi, r.lo, i.lo);
@@ -439,14 +454,23 @@ struct ADF {
   static QS_HD store_t to_store_f(reg_t v, bool df) { return df ? to_df(v) : to_store(v); }
   static QS_HD reg_t zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
+  // U x + V y lane-wise for double-float patterns, U given by its high part and the negated
+  // parts, V by its parts; the two products' low-order terms run in two chains
+  static QS_HD reg_t dot2(float2 Uh, float2 nUh, float2 nUl, float2 xh, float2 xl, float2 Vh, float2 Vl, float2 yh,
+                          float2 yl) {
+    const float2 p = mul2(Uh, xh);
+    float2 n = fma2(nUh, xh, p);             // -(rounding error of p), exact
+    n = fma2(nUh, xl, n);
+    n = fma2(nUl, xh, n);
+    float2 s, d, c;
+    add_prod2(p, Vh, yh, s, d, c);
+    d = fma2(Vh, yl, d);
+    d = fma2(Vl, yh, d);
+    return mk(s, add2(c, sub2(d, n)));
+  }
   // u a
   static QS_HD reg_t mul(const mat_t& u, reg_t a) {
-    float2 p1, n1, p2, n2, s, e;
-    prod2(make_float2(u.a.x, u.a.y), make_float2(u.a.z, u.a.w), make_float2(u.c.x, u.c.y), hi(a), lo(a), p1, n1);
-    prod2(make_float2(u.b.x, u.b.y), make_float2(u.b.z, u.b.w), make_float2(u.c.z, u.c.w), swp(hi(a)), swp(lo(a)),
-          p2, n2);
-    two_sum2(p1, p2, s, e);
-    return mk(s, sub2(e, add2(n1, n2)));
+    return dot2(mA(u), mnA(u), mnAl(u), hi(a), lo(a), mB(u), mBl(u), swp(hi(a)), swp(lo(a)));
   }
   static QS_HD reg_t add(reg_t x, reg_t y) {
     float2 s, e;
@@ -454,55 +478,46 @@ struct ADF {
     return mk(s, add2(e, add2(lo(x), lo(y))));
   }
   // acc + u a
-  static QS_HD reg_t mac(reg_t acc, const mat_t& u, reg_t a) { return add(acc, mul(u, a)); }
+  static QS_HD reg_t mac(reg_t acc, const mat_t& u, reg_t a) {
+    float2 s, d, c, s2, d2, c2;
+    const float2 as = swp(hi(a));
+    add_prod2(hi(acc), mA(u), hi(a), s, d, c);
+    add_prod2(s, mB(u), as, s2, d2, c2);
+    d = fma2(mA(u), lo(a), d);
+    d = fma2(mAl(u), hi(a), d);
+    d2 = fma2(mB(u), swp(lo(a)), d2);
+    d2 = fma2(mBl(u), as, d2);
+    return mk(s2, add2(lo(acc), add2(add2(c, d), add2(c2, d2))));
+  }
   // u a + v b
   static QS_HD reg_t mac2(const mat_t& u, reg_t a, const mat_t& v, reg_t b) { return add(mul(u, a), mul(v, b)); }
   // c a - i s b for cs = (c, s), plain frame: c (.) a + (s, -s) (.) swap(b), and (s, -s) is
   // the negated (-ui, ui) pattern of the entry
   static QS_HD reg_t rx(const mat_t& cs, reg_t a, reg_t b) {
-    float2 p1, n1, p2, n2, s, e;
-    prod2(make_float2(cs.a.x, cs.a.y), make_float2(cs.a.z, cs.a.w), make_float2(cs.c.x, cs.c.y), hi(a), lo(a), p1, n1);
-    prod2(make_float2(cs.b.x, cs.b.y), make_float2(cs.b.z, cs.b.w), make_float2(cs.c.z, cs.c.w), swp(hi(b)),
-          swp(lo(b)), p2, n2);
-    two_diff2(p1, p2, s, e);   // (p1 - n1) - (p2 - n2)
-    return mk(s, add2(e, sub2(n2, n1)));
+    return dot2(mA(cs), mnA(cs), mnAl(cs), hi(a), lo(a), neg2(mB(cs)), neg2(mBl(cs)), swp(hi(b)), swp(lo(b)));
   }
 
   // ---- phase-frame updates with a real double-float factor t
+  // u + (th + tl) v
+  static QS_HD reg_t add_prod(float2 th, float2 tl, reg_t v, float2 uh, float2 ul) {
+    float2 s, d, c;
+    add_prod2(uh, th, hi(v), s, d, c);
+    d = fma2(th, lo(v), d);
+    d = fma2(tl, hi(v), d);
+    return mk(s, add2(ul, add2(c, d)));
+  }
   // u + t v
-  static QS_HD reg_t axpy_r(const dfr& t, reg_t v, reg_t u) {
-    float2 p, n, s, e;
-    prod2(t.h, t.nh, t.nl, hi(v), lo(v), p, n);
-    two_sum2(hi(u), p, s, e);
-    return mk(s, add2(e, sub2(lo(u), n)));
-  }
+  static QS_HD reg_t axpy_r(const dfr& t, reg_t v, reg_t u) { return add_prod(t.h, t.l, v, hi(u), lo(u)); }
   // u - t v
-  static QS_HD reg_t axmy_r(const dfr& t, reg_t v, reg_t u) {
-    float2 p, n, s, e;
-    prod2(t.h, t.nh, t.nl, hi(v), lo(v), p, n);
-    two_diff2(hi(u), p, s, e);
-    return mk(s, add2(e, add2(lo(u), n)));
-  }
+  static QS_HD reg_t axmy_r(const dfr& t, reg_t v, reg_t u) { return add_prod(t.nh, t.nl, v, hi(u), lo(u)); }
   // t v - u
   static QS_HD reg_t ymx_r(const dfr& t, reg_t v, reg_t u) {
-    float2 p, n, s, e;
-    prod2(t.h, t.nh, t.nl, hi(v), lo(v), p, n);
-    two_diff2(p, hi(u), s, e);
-    return mk(s, sub2(e, add2(n, lo(u))));
+    return add_prod(t.h, t.l, v, neg2(hi(u)), neg2(lo(u)));
   }
   // (a, b) -> (c a + s b, c b - s a) with real c and s
   static QS_HD void rot_r(const dfr& c, const dfr& sn, reg_t a, reg_t b, reg_t& a2, reg_t& b2) {
-    const float2 ch = c.h, nch = c.nh, ncl = c.nl;
-    const float2 sh = sn.h, nsh = sn.nh, nsl = sn.nl;
-    float2 p1, n1, p2, n2, s, e;
-    prod2(ch, nch, ncl, hi(a), lo(a), p1, n1);
-    prod2(sh, nsh, nsl, hi(b), lo(b), p2, n2);
-    two_sum2(p1, p2, s, e);
-    const reg_t ra = mk(s, sub2(e, add2(n1, n2)));
-    prod2(ch, nch, ncl, hi(b), lo(b), p1, n1);
-    prod2(sh, nsh, nsl, hi(a), lo(a), p2, n2);
-    two_diff2(p1, p2, s, e);
-    b2 = mk(s, add2(e, sub2(n2, n1)));
+    const reg_t ra = dot2(c.h, c.nh, c.nl, hi(a), lo(a), sn.h, sn.l, hi(b), lo(b));
+    b2 = dot2(c.h, c.nh, c.nl, hi(b), lo(b), sn.nh, sn.nl, hi(a), lo(a));
     a2 = ra;
   }
   // v (-i)^q, exact (a lane swap and sign flips); q in 0..3

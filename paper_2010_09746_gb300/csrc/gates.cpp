@@ -142,7 +142,7 @@ void Pool::serialise_into(Policy pol, unsigned char* dst) const {
     memcpy(dst, f64.data(), E * 16);
   } else {
     // double-float lane patterns of u = ur + i ui (12 floats): (ur, ur) and its negation,
-    // (-ui, ui) and its negation, then the negated low parts of (ur, ur) and (-ui, ui)
+    // (-ui, ui) and the low part of (ur, ur), the low part of (-ui, ui) and that of (-ur, -ur)
     float* f = (float*)dst;
     for (size_t k = 0; k < E; k++) {
       const double ur = f64[2 * k], ui = f64[2 * k + 1];
@@ -150,8 +150,8 @@ void Pool::serialise_into(Policy pol, unsigned char* dst) const {
       const float ih = (float)ui, il = (float)(ui - (double)ih);
       float* e = f + 12 * k;
       e[0] = rh; e[1] = rh; e[2] = -rh; e[3] = -rh;
-      e[4] = -ih; e[5] = ih; e[6] = ih; e[7] = -ih;
-      e[8] = -rl; e[9] = -rl; e[10] = il; e[11] = -il;
+      e[4] = -ih; e[5] = ih; e[6] = rl; e[7] = rl;
+      e[8] = -il; e[9] = il; e[10] = -rl; e[11] = -rl;
     }
   }
 }
