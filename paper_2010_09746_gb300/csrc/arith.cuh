@@ -535,4 +535,10 @@ struct ADF {
   }
 };
 
+// one host matrix entry, (re, im) in double, in a policy's format (df_entry: gates.cpp)
+void df_entry(const double* z, float* e);
+inline void host_entry(const double* z, float2* m) { *m = make_float2((float)z[0], (float)z[1]); }
+inline void host_entry(const double* z, double2* m) { *m = make_double2(z[0], z[1]); }
+inline void host_entry(const double* z, dfm* m) { df_entry(z, (float*)m); }
+
 }  // namespace qs

@@ -175,7 +175,11 @@ qs_status apply_hgate(qs_state* h, const HGate& g) {
   ctx.tile = false;
   if (!lower_gate(g, ctx, pool, ops)) return fail(QS_EINVAL, "gate could not be lowered");
   const Policy pol = policy_for(h->dtype, h->arith);
-  std::vector<unsigned char> ser = pool.serialise(pol);
+  // small matrices are kernel parameters; only the largest blocks read theirs from device memory
+  bool needs_pool = false;
+  for (const DevOp& o : ops) needs_pool |= gate_needs_pool(pol, o);
+  std::vector<unsigned char> ser;
+  if (needs_pool) ser = pool.serialise(pol);
   if (ser.size() > h->gate_pool_bytes) {
     dev_free_as(h->gate_pool, h->gate_pool_bytes, h->stream, h->native_alloc);
     h->gate_pool_bytes = std::max<size_t>(ser.size(), 64 * 1024);
@@ -187,7 +191,7 @@ qs_status apply_hgate(qs_state* h, const HGate& g) {
   for (const DevOp& o : ops) {
     Step s;
     s.kind = ST_GATE;
-    CUDA_TRY(timed(h, step_name(s, pol), 0.0, [&] { return launch_gate(pol, h->psi, h->n, o, h->gate_pool, h->stream); }),
+    CUDA_TRY(timed(h, step_name(s, pol), 0.0, [&] { return launch_gate(pol, h->psi, h->n, o, pool.f64.data(), h->gate_pool, h->stream); }),
              "gate launch");
   }
   return QS_OK;
@@ -705,7 +709,8 @@ static qs_status execute_steps(qs_handle h, qs_plan_t p) {
         h->sigma = s.perm;
       }
     } else if (s.kind == ST_GATE) {
-      CUDA_TRY(timed(h, name, s.bytes, [&] { return launch_gate(p->pol, h->psi, h->n, s.op, p->pool_dev, h->stream); },
+      CUDA_TRY(timed(h, name, s.bytes,
+                     [&] { return launch_gate(p->pol, h->psi, h->n, s.op, p->cr.pool.f64.data(), p->pool_dev, h->stream); },
                      s.alu),
                "gate launch");
     } else if (s.kind == ST_RENORM) {

@@ -130,6 +130,17 @@ HGate make_1q_gate(int q, const cd m[4]) {
 
 size_t Pool::entry_bytes(Policy pol) { return pol == POL_F32 ? 8 : (pol == POL_F64 ? 16 : 48); }
 
+// double-float lane patterns of u = ur + i ui (12 floats): (ur, ur) and its negation, (-ui, ui)
+// and the low part of (ur, ur), the low part of (-ui, ui) and that of (-ur, -ur)
+void df_entry(const double* z, float* e) {
+  const double ur = z[0], ui = z[1];
+  const float rh = (float)ur, rl = (float)(ur - (double)rh);
+  const float ih = (float)ui, il = (float)(ui - (double)ih);
+  e[0] = rh; e[1] = rh; e[2] = -rh; e[3] = -rh;
+  e[4] = -ih; e[5] = ih; e[6] = rl; e[7] = rl;
+  e[8] = -il; e[9] = il; e[10] = -rl; e[11] = -rl;
+}
+
 void Pool::serialise_into(Policy pol, unsigned char* dst) const {
   const size_t E = entries();
   if (pol == POL_F32) {
@@ -141,18 +152,8 @@ void Pool::serialise_into(Policy pol, unsigned char* dst) const {
   } else if (pol == POL_F64) {
     memcpy(dst, f64.data(), E * 16);
   } else {
-    // double-float lane patterns of u = ur + i ui (12 floats): (ur, ur) and its negation,
-    // (-ui, ui) and the low part of (ur, ur), the low part of (-ui, ui) and that of (-ur, -ur)
     float* f = (float*)dst;
-    for (size_t k = 0; k < E; k++) {
-      const double ur = f64[2 * k], ui = f64[2 * k + 1];
-      const float rh = (float)ur, rl = (float)(ur - (double)rh);
-      const float ih = (float)ui, il = (float)(ui - (double)ih);
-      float* e = f + 12 * k;
-      e[0] = rh; e[1] = rh; e[2] = -rh; e[3] = -rh;
-      e[4] = -ih; e[5] = ih; e[6] = rl; e[7] = rl;
-      e[8] = -il; e[9] = il; e[10] = -rl; e[11] = -rl;
-    }
+    for (size_t k = 0; k < E; k++) df_entry(&f64[2 * k], f + 12 * k);
   }
 }
 

@@ -53,26 +53,18 @@ int grid_for(uint64_t work) {
   return (int)blocks;
 }
 
+// The one to four matrix entries of a gate travel as a kernel parameter: constant-bank operands, and
+// nothing to upload before the launch.
 template <class A>
-__global__ void __launch_bounds__(kThreads) k_u1(typename A::store_t* __restrict__ psi, uint64_t nwork,
-                                                 Expand e, int p, const typename A::mat_t* __restrict__ m) {
-  using R = typename A::reg_t;
-  const typename A::mat_t u00 = m[0], u01 = m[1], u10 = m[2], u11 = m[3];
-  const uint64_t s = 1ull << p;
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t i0 = expand(t, e);
-    R a = A::from_store(psi[i0]);
-    R b = A::from_store(psi[i0 | s]);
-    psi[i0] = A::to_store(A::mac2(u00, a, u01, b));
-    psi[i0 | s] = A::to_store(A::mac2(u10, a, u11, b));
-  }
-}
+struct GateMat {
+  typename A::mat_t u[4];
+};
 
 template <class A>
 __global__ void __launch_bounds__(kThreads) k_rx(typename A::store_t* __restrict__ psi, uint64_t nwork,
-                                                 Expand e, int p, const typename A::mat_t* __restrict__ m) {
+                                                 Expand e, int p, const __grid_constant__ GateMat<A> m) {
   using R = typename A::reg_t;
-  const typename A::mat_t cs = m[0];
+  const typename A::mat_t cs = m.u[0];
   const uint64_t s = 1ull << p;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t i0 = expand(t, e);
@@ -86,8 +78,8 @@ __global__ void __launch_bounds__(kThreads) k_rx(typename A::store_t* __restrict
 // diag(d0, d1) on bit p, amplitudes with the control bits set
 template <class A>
 __global__ void __launch_bounds__(kThreads) k_diag(typename A::store_t* __restrict__ psi, uint64_t nwork,
-                                                   Expand e, int p, const typename A::mat_t* __restrict__ m) {
-  const typename A::mat_t d0 = m[0], d1 = m[1];
+                                                   Expand e, int p, const __grid_constant__ GateMat<A> m) {
+  const typename A::mat_t d0 = m.u[0], d1 = m.u[1];
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t i = expand(t, e);
     psi[i] = A::to_store(A::mul(((i >> p) & 1) ? d1 : d0, A::from_store(psi[i])));
@@ -97,8 +89,8 @@ __global__ void __launch_bounds__(kThreads) k_diag(typename A::store_t* __restri
 // multiply by d0 on the amplitudes whose fixed bits (the inserted positions) are all one
 template <class A>
 __global__ void __launch_bounds__(kThreads) k_phase(typename A::store_t* __restrict__ psi, uint64_t nwork,
-                                                    Expand e, const typename A::mat_t* __restrict__ m) {
-  const typename A::mat_t d = m[0];
+                                                    Expand e, const __grid_constant__ GateMat<A> m) {
+  const typename A::mat_t d = m.u[0];
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t i = expand(t, e);
     psi[i] = A::to_store(A::mul(d, A::from_store(psi[i])));
@@ -135,9 +127,9 @@ __global__ void __launch_bounds__(kThreads) k_exchange(S* __restrict__ psi, uint
 // pairs.  Controls never include bit 0 here (the launcher falls back otherwise).
 template <bool kRX>
 __global__ void __launch_bounds__(kThreads) k_pair_c64x2(float2* __restrict__ psi, uint64_t nwork, Expand e, int p,
-                                                          const float2* __restrict__ m) {
+                                                          const __grid_constant__ GateMat<AF32> m) {
   using A = AF32;
-  const float2 u00 = m[0], u01 = kRX ? m[0] : m[1], u10 = kRX ? m[0] : m[2], u11 = kRX ? m[0] : m[3];
+  const float2 u00 = m.u[0], u01 = kRX ? m.u[0] : m.u[1], u10 = kRX ? m.u[0] : m.u[2], u11 = kRX ? m.u[0] : m.u[3];
   float4* psi4 = reinterpret_cast<float4*>(psi);
   const uint64_t s = 1ull << p;
   auto upd = [&](float2 a, float2 b, float2& ra, float2& rb) {
@@ -171,11 +163,11 @@ __global__ void __launch_bounds__(kThreads) k_pair_c64x2(float2* __restrict__ ps
 // control): kind 0 = diag(d0, d1) on bit p, 1 = multiply by d0, 2 = exact sign flip
 template <int kKind>
 __global__ void __launch_bounds__(kThreads) k_diag_c64x2(float2* __restrict__ psi, uint64_t nwork, Expand e, int p,
-                                                          const float2* __restrict__ m) {
+                                                          const __grid_constant__ GateMat<AF32> m) {
   using A = AF32;
   float4* psi4 = reinterpret_cast<float4*>(psi);
-  const float2 d0 = kKind == 2 ? make_float2(0.f, 0.f) : m[0];
-  const float2 d1 = kKind == 0 ? m[1] : d0;
+  const float2 d0 = kKind == 2 ? make_float2(0.f, 0.f) : m.u[0];
+  const float2 d1 = kKind == 0 ? m.u[1] : d0;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t i = expand(t, e);
     float4 v = psi4[i >> 1];
@@ -194,7 +186,8 @@ __global__ void __launch_bounds__(kThreads) k_diag_c64x2(float2* __restrict__ ps
   }
 }
 
-// dense 2^K x 2^K on bits kq[0..K-1]: a block stages kThreads / 2^K groups of 2^K
+// dense 2^K x 2^K on bits kq[0..K-1] for the blocks too large for registers (K = 6, and K = 5 of
+// complex128), the matrix in global memory: a block stages kThreads / 2^K groups of 2^K
 // amplitudes in shared memory; thread (g, r) computes output row r of group g.
 template <class A, int K>
 __global__ void __launch_bounds__(kThreads) k_dense(typename A::store_t* __restrict__ psi, uint64_t nwork,
@@ -240,7 +233,7 @@ Expand make_expand(int n, uint64_t zero_bits, uint64_t ones, uint64_t* nwork) {
 }
 
 // complex64 gates that the 16-byte kernels cover; false = use the general kernels
-bool launch_gate_c64x2(float2* psi, int n, const DevOp& op, const float2* mp, cudaStream_t st) {
+bool launch_gate_c64x2(float2* psi, int n, const DevOp& op, const GateMat<AF32>& mp, cudaStream_t st) {
   if (n < 2 || (op.cmask & 1ull) || __builtin_popcountll(op.cmask) > 6) return false;
   uint64_t nwork = 0;
   switch (op.type) {
@@ -268,21 +261,28 @@ bool launch_gate_c64x2(float2* psi, int n, const DevOp& op, const float2* mp, cu
   }
 }
 
+// entries an op's kernel takes as parameters
+int param_entries(const DevOp& op) {
+  if (op.mat < 0) return 0;
+  return op.type == OP_DIAG ? 2 : (op.type == OP_U1 ? 4 : (op.type == OP_RX || op.type == OP_PHASE ? 1 : 0));
+}
+
 template <class A>
-cudaError_t launch_gate_t(void* psi_v, int n, const DevOp& op, const void* pool, cudaStream_t st) {
+cudaError_t launch_gate_t(Policy pol, void* psi_v, int n, const DevOp& op, const double* entries, const void* pool,
+                          cudaStream_t st) {
   using S = typename A::store_t;
   using M = typename A::mat_t;
   S* psi = (S*)psi_v;
-  const M* mp = (const M*)pool + op.mat;
+  GateMat<A> mp{};
+  for (int k = 0; k < param_entries(op); k++) host_entry(entries + 2 * ((size_t)op.mat + k), &mp.u[k]);
   uint64_t nwork = 0;
   if constexpr (std::is_same<A, AF32>::value) {   // complex64: 16-byte accesses where possible
     if (launch_gate_c64x2(psi, n, op, mp, st)) return cudaGetLastError();
   }
   switch (op.type) {
     case OP_U1: {
-      Expand e = make_expand(n, 1ull << op.k0, op.cmask, &nwork);
-      k_u1<A><<<grid_for(nwork), kThreads, 0, st>>>(psi, nwork, e, op.k0, mp);
-      break;
+      const int q = op.k0;
+      return launch_block(pol, psi, n, 1, &q, op.cmask, entries + 2 * (size_t)op.mat, st);
     }
     case OP_RX: {
       Expand e = make_expand(n, 1ull << op.k0, op.cmask, &nwork);
@@ -295,13 +295,9 @@ cudaError_t launch_gate_t(void* psi_v, int n, const DevOp& op, const void* pool,
       break;
     }
     case OP_PHASE: {
-      if (op.mat < 0) {   // exact -1
-        Expand e = make_expand(n, 0, op.cmask, &nwork);
-        k_negate<S><<<grid_for(nwork), kThreads, 0, st>>>(psi, nwork, e);
-      } else {
-        Expand e = make_expand(n, 0, op.cmask, &nwork);
-        k_phase<A><<<grid_for(nwork), kThreads, 0, st>>>(psi, nwork, e, mp);
-      }
+      Expand e = make_expand(n, 0, op.cmask, &nwork);
+      if (op.mat < 0) k_negate<S><<<grid_for(nwork), kThreads, 0, st>>>(psi, nwork, e);   // exact -1
+      else k_phase<A><<<grid_for(nwork), kThreads, 0, st>>>(psi, nwork, e, mp);
       break;
     }
     case OP_X: {
@@ -322,17 +318,19 @@ cudaError_t launch_gate_t(void* psi_v, int n, const DevOp& op, const void* pool,
         o.kq[0] = op.k0;
         o.kq[1] = op.k1;
       }
+      if (block_supported(pol, o.nk, o.cmask))
+        return launch_block(pol, psi, n, o.nk, o.kq, o.cmask, entries + 2 * (size_t)op.mat, st);
+      if (!pool) return cudaErrorInvalidValue;
+      const M* dm = (const M*)pool + op.mat;
       uint64_t zb = 0;
       for (int t = 0; t < o.nk; t++) zb |= 1ull << o.kq[t];
       Expand e = make_expand(n, zb, op.cmask, &nwork);
       const int g = grid_for(nwork << o.nk);
       switch (o.nk) {
-        case 1: k_dense<A, 1><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
-        case 2: k_dense<A, 2><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
-        case 3: k_dense<A, 3><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
-        case 4: k_dense<A, 4><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
-        case 5: k_dense<A, 5><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
-        case 6: k_dense<A, 6><<<g, kThreads, 0, st>>>(psi, nwork, e, o, mp); break;
+        case 5:
+          if constexpr (!std::is_same<A, AF32>::value) k_dense<A, 5><<<g, kThreads, 0, st>>>(psi, nwork, e, o, dm);
+          break;
+        case 6: k_dense<A, 6><<<g, kThreads, 0, st>>>(psi, nwork, e, o, dm); break;
         default: return cudaErrorInvalidValue;
       }
       break;
@@ -507,11 +505,16 @@ cudaError_t launch_batch_norms(const void* psi, int is_c128, const uint64_t* off
   return cudaGetLastError();
 }
 
-cudaError_t launch_gate(Policy pol, void* psi, int n, const DevOp& op, const void* pool, cudaStream_t s) {
+bool gate_needs_pool(Policy pol, const DevOp& op) {
+  return op.type == OP_DENSE && !block_supported(pol, op.nk, op.cmask);
+}
+
+cudaError_t launch_gate(Policy pol, void* psi, int n, const DevOp& op, const double* entries, const void* pool,
+                        cudaStream_t s) {
   switch (pol) {
-    case POL_F32: return launch_gate_t<AF32>(psi, n, op, pool, s);
-    case POL_F64: return launch_gate_t<AF64>(psi, n, op, pool, s);
-    case POL_DF: return launch_gate_t<ADF>(psi, n, op, pool, s);
+    case POL_F32: return launch_gate_t<AF32>(pol, psi, n, op, entries, pool, s);
+    case POL_F64: return launch_gate_t<AF64>(pol, psi, n, op, entries, pool, s);
+    case POL_DF: return launch_gate_t<ADF>(pol, psi, n, op, entries, pool, s);
   }
   return cudaErrorInvalidValue;
 }

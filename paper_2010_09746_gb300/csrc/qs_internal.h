@@ -128,7 +128,16 @@ struct Step {
 // launch.  `pool` is a device array of policy-format matrix entries.
 // ------------------------------------------------------------------------------------------
 cudaError_t launch_init_zero(void* psi, int n, int store_bytes, cudaStream_t s);
-cudaError_t launch_gate(Policy pol, void* psi, int n, const DevOp& op, const void* pool, cudaStream_t s);
+// entries: the pool's (re, im) pairs on the host (the kernels take small matrices as parameters);
+// pool: its device copy in the policy's format, used only where gate_needs_pool says so
+cudaError_t launch_gate(Policy pol, void* psi, int n, const DevOp& op, const double* entries, const void* pool,
+                        cudaStream_t s);
+bool gate_needs_pool(Policy pol, const DevOp& op);
+// dense 2^k x 2^k matrix u ((re, im) pairs, row-major, host) on storage bits kq[0..k-1] where the
+// bits of ctl are 1; for the sizes block_supported accepts
+bool block_supported(Policy pol, int k, uint64_t ctl);
+cudaError_t launch_block(Policy pol, void* psi, int n, int k, const int* kq, uint64_t ctl, const double* u,
+                         cudaStream_t s);
 // reads the state at psi, writes it to dst (the same buffer unless the pass carries a fused
 // permutation, tp.swap_a != tp.swap_b)
 cudaError_t launch_tile_pass(Policy pol, const void* psi, void* dst, const TilePass& tp, const StageRec* stages_dev,
@@ -198,6 +207,9 @@ struct FuseOrigin {
   int count(size_t i) const { return off[i + 1] - off[i]; }
 };
 void fuse_single_qubit_runs(int n, std::vector<HGate>& in, std::vector<HGate>* out, FuseOrigin* origin);
+// one matrix entry, (re, im) in double, as the 12 floats of the double-float lane patterns
+void df_entry(const double* z, float* e);
+
 // Matrix pool in policy format.
 struct Pool {
   std::vector<double> f64;  // (re, im) pairs
