@@ -142,13 +142,87 @@ bool is_identity(const cd m[4]) { return m[0] == cd(1, 0) && m[1] == cd(0, 0) &&
 // with the other register qubits.  So a run is fused when it holds two or more non-diagonal
 // gates, or a general one (neither RX nor X in form), or consists of diagonal gates only (one
 // diagonal factor).  A run whose one non-diagonal gate is an RX or an X is kept as it is.
-void fuse_single_qubit_runs(int n, std::vector<HGate>& in, std::vector<HGate>* out, FuseOrigin* origin) {
+//
+// A CNOT whose target has such a general run directly before and directly after it is fused
+// as H . CZ . H with the two Hadamards multiplied into those runs, which cost a product
+// either way; several CNOTs onto one target with nothing in between share the two Hadamards.
+// A CZ is diagonal: it needs no qubit in the tile or in registers, so passes and stages hold
+// more gates, and inside a stage it joins the phase tables instead of moving amplitudes
+// (a 23-qubit circuit of 50 layers of Haar gates and CNOT / CZ: 39 -> 35 passes, 138 -> 126
+// stages, 1781 -> 1307 register ops, 20.0 -> 16.4 ms; 12 qubits, 20 layers of CNOT: 574 -> 395 us).
+// It changes the products' rounding, so it is done where that stays below what the state's
+// type resolves in its FP64 read-outs: complex128 (cz_form); complex64 plans, whose norms and
+// probabilities would move by 1e-7, keep the CNOT.
+namespace {
+
+// shape of the single-qubit gates between two multi-qubit gates on a qubit
+struct RunShape {
+  int nd = 0;             // non-diagonal gates
+  bool general = false;   // one that is neither RX nor X in form
+  int size = 0;
+  void add(const HGate& g) {
+    size++;
+    if (g.cls[0] == CLS_Z) return;
+    nd++;
+    const cd* m = g.U.data();
+    const bool x_form = m[0] == cd(0, 0) && m[3] == cd(0, 0) && m[1] == cd(1, 0) && m[2] == cd(1, 0);
+    const bool rx_form = m[0] == m[3] && m[0].imag() == 0.0 && m[1] == m[2] && m[1].real() == 0.0;
+    general |= !x_form && !rx_form;
+  }
+  bool product() const { return general || nd >= 2; }   // runs as diag . RX . diag whatever it is
+};
+
+// which CNOTs fuse as H . CZ . H: per target qubit, maximal sequences of CNOTs onto it with no
+// other gate on it in between, bounded by a run of the product kind on either side
+std::vector<char> cnots_to_cz(int n, const std::vector<HGate>& in) {
+  std::vector<char> conv(in.size(), 0);
+  struct Q {
+    RunShape run;                // since the last multi-qubit gate
+    std::vector<int> open;       // CNOTs onto this qubit whose run after is not known yet
+  };
+  std::vector<Q> qs(n);
+  for (int i = 0; i < (int)in.size(); i++) {
+    const HGate& g = in[i];
+    if (g.nq == 1) {
+      qs[g.q[0]].run.add(g);
+      continue;
+    }
+    for (int t = 0; t < g.nq; t++) {
+      Q& s = qs[g.q[t]];
+      const bool onto = g.kind == QS_OP_CNOT && t == 1;
+      if (!s.open.empty() && s.run.size > 0) {   // the sequence ended with this run
+        if (s.run.product())
+          for (int k : s.open) conv[k] = 1;
+        s.open.clear();
+      } else if (!s.open.empty() && !onto) {     // another gate right after it: no run to fuse into
+        s.open.clear();
+      }
+      if (onto && (s.run.product() || !s.open.empty())) s.open.push_back(i);
+      s.run = RunShape();
+    }
+  }
+  for (Q& s : qs)
+    if (s.run.product())
+      for (int k : s.open) conv[k] = 1;
+  return conv;
+}
+
+}  // namespace
+
+void fuse_single_qubit_runs(int n, std::vector<HGate>& in, bool cz_form, std::vector<HGate>* out, FuseOrigin* origin) {
   out->clear();
   out->reserve(in.size());
   origin->off.assign(1, 0);
   origin->idx.clear();
   origin->idx.reserve(in.size());
+  // a run's gates in order; kHadamard stands for a Hadamard of a CNOT fused as H . CZ . H
+  constexpr int kHadamard = -1;
+  const double rh = std::sqrt(0.5);
+  const cd H[4] = {rh, rh, rh, -rh};
+  std::vector<char> to_cz(in.size(), 0);
+  if (cz_form) to_cz = cnots_to_cz(n, in);
   std::vector<std::vector<int>> run(n);
+  std::vector<int> real;
   auto close = [&] { origin->off.push_back((int)origin->idx.size()); };
   auto keep = [&](int i) {   // an input gate as it is (moved: the input is consumed)
     out->push_back(std::move(in[i]));
@@ -163,40 +237,49 @@ void fuse_single_qubit_runs(int n, std::vector<HGate>& in, std::vector<HGate>* o
   auto flush = [&](int q) {
     std::vector<int>& r = run[q];
     if (r.empty()) return;
-    int nd = 0;
-    bool general = false;
+    RunShape shape;
+    real.clear();
     for (int i : r) {
-      if (in[i].cls[0] == CLS_Z) continue;
-      nd++;
-      const cd* m = in[i].U.data();
-      const bool x_form = m[0] == cd(0, 0) && m[3] == cd(0, 0) && m[1] == cd(1, 0) && m[2] == cd(1, 0);
-      const bool rx_form = m[0] == m[3] && m[0].imag() == 0.0 && m[1] == m[2] && m[1].real() == 0.0;
-      general |= !x_form && !rx_form;
+      if (i == kHadamard) continue;
+      shape.add(in[i]);
+      real.push_back(i);
     }
-    if (r.size() < 2 || (nd == 1 && !general)) {   // a lone general gate splits at lowering
+    const bool all_real = real.size() == r.size();
+    if (all_real && (r.size() < 2 || (shape.nd == 1 && !shape.general))) {   // a lone general gate splits at lowering
       for (int i : r) keep(i);
       r.clear();
       return;
     }
     cd U[4] = {1, 0, 0, 1}, t[4];
-    for (int i : r) {   // later gates act on the left
-      const cd G[4] = {in[i].U[0], in[i].U[1], in[i].U[2], in[i].U[3]};
+    for (size_t k = 0; k < r.size(); k++) {   // later gates act on the left
+      if (r[k] == kHadamard && k + 1 < r.size() && r[k + 1] == kHadamard) {   // between two CNOTs: H H = 1
+        k++;
+        continue;
+      }
+      cd G[4];
+      for (int e = 0; e < 4; e++) G[e] = r[k] == kHadamard ? H[e] : in[r[k]].U[e];
       mul2x2(G, U, t);
-      for (int k = 0; k < 4; k++) U[k] = t[k];
+      for (int e = 0; e < 4; e++) U[e] = t[e];
+    }
+    if (real.empty() && is_identity(U)) {   // two Hadamards that cancelled: no gate is left
+      r.clear();
+      return;
     }
     // the product as separate gates diag, RX, diag: the scheduler may then place the two
     // diagonal factors wherever their phase tables are cheapest
     cd d1[4], rx[4], d2[4];
-    if (is_identity(U)) {
+    if (is_identity(U) && all_real) {
       for (int i : r) keep(i);   // an exact identity: keep the gates (rare)
     } else if (U[1] == cd(0, 0) && U[2] == cd(0, 0)) {
-      emit(make_1q_gate(q, U), r);
+      emit(make_1q_gate(q, U), real);
+    } else if (real.size() == 1) {   // one gate and Hadamards: as a lone general gate, it splits at lowering
+      emit(make_1q_gate(q, U), real);
     } else if (euler_split(U, d1, rx, d2)) {
       if (!is_identity(d1)) emit(make_1q_gate(q, d1), {});
-      emit(make_1q_gate(q, rx), r);
+      emit(make_1q_gate(q, rx), real);
       if (!is_identity(d2)) emit(make_1q_gate(q, d2), {});
     } else {
-      emit(make_1q_gate(q, U), r);
+      emit(make_1q_gate(q, U), real);
     }
     r.clear();
   };
@@ -204,6 +287,23 @@ void fuse_single_qubit_runs(int n, std::vector<HGate>& in, std::vector<HGate>* o
     const HGate& g = in[i];
     if (g.nq == 1) {
       run[g.q[0]].push_back(i);
+      continue;
+    }
+    if (to_cz[i]) {
+      const int c = g.q[0], t = g.q[1];
+      run[t].push_back(kHadamard);
+      flush(c);
+      flush(t);
+      qs_op op{};
+      op.kind = QS_OP_CZ;
+      op.nq = 2;
+      op.q[0] = c;
+      op.q[1] = t;
+      op.mat = -1;
+      std::string err;
+      make_hgate(n, op, nullptr, 0, &in[i], &err);   // a valid gate: both qubits were checked
+      keep(i);
+      run[t].push_back(kHadamard);
       continue;
     }
     for (int t = 0; t < g.nq; t++) flush(g.q[t]);
@@ -808,7 +908,7 @@ bool compile_circuit(int n, std::vector<HGate> gates, const std::vector<int>& si
     } else {
       std::vector<HGate> fused;
       FuseOrigin origin;
-      fuse_single_qubit_runs(n, gates, &fused, &origin);   // consumes gates
+      fuse_single_qubit_runs(n, gates, out->pol != POL_F32, &fused, &origin);   // consumes gates
       ok = compile_tile(n, fused, sigma0, o, store_bytes, out, err, &origin);
       for (size_t i = 0; i < fused.size(); i++)
         if (origin.count(i) >= 2) out->stats.n_fused += origin.count(i);

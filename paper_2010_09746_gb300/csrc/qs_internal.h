@@ -201,12 +201,13 @@ bool euler_split(const cd U[4], cd d1[4], cd rx[4], cd d2[4]);
 // re-expressed as at most three gates
 // (diagonal, RX, diagonal).  The origin lists the input gates each output gate stands for
 // (empty for the extra factors of a product); every input gate appears exactly once.  The
-// input gates are moved into the output (`in` is consumed).
+// input gates are moved into the output (`in` is consumed).  cz_form: a CNOT whose target has such
+// runs on either side becomes H . CZ . H, its Hadamards part of the runs.
 struct FuseOrigin {
   std::vector<int> off, idx;   // output gate i stands for input gates idx[off[i] .. off[i + 1])
   int count(size_t i) const { return off[i + 1] - off[i]; }
 };
-void fuse_single_qubit_runs(int n, std::vector<HGate>& in, std::vector<HGate>* out, FuseOrigin* origin);
+void fuse_single_qubit_runs(int n, std::vector<HGate>& in, bool cz_form, std::vector<HGate>* out, FuseOrigin* origin);
 // one matrix entry, (re, im) in double, as the 12 floats of the double-float lane patterns
 void df_entry(const double* z, float* e);
 
