@@ -420,6 +420,15 @@ struct ADF {
     return dfr{make_float2(m.a.x, m.a.y), make_float2(m.a.z, m.a.w), make_float2(m.b.z, m.b.w),
                make_float2(m.c.z, m.c.w)};
   }
+  // an entry as an amplitude and back (its own lane patterns of a value that is not normalised)
+  static QS_HD reg_t from_mat(const mat_t& m) { return make_float4(m.a.x, m.b.y, m.b.z, m.c.y); }
+  static QS_HD mat_t to_mat(reg_t v) {
+    mat_t m;
+    m.a = make_float4(v.x, v.x, -v.x, -v.x);
+    m.b = make_float4(-v.y, v.y, v.z, v.z);
+    m.c = make_float4(-v.w, v.w, -v.z, -v.z);
+    return m;
+  }
   // the lane patterns of an entry
   static QS_HD float2 mA(const mat_t& m) { return make_float2(m.a.x, m.a.y); }     // ( ur,  ur)
   static QS_HD float2 mnA(const mat_t& m) { return make_float2(m.a.z, m.a.w); }    // (-ur, -ur)

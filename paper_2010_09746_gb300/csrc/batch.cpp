@@ -146,8 +146,9 @@ qs_status batch_from_plans(const std::vector<const qs_plan*>& plans, qs_dtype dt
           st.op0 += (st.kind == 0) ? rbase[i] : dbase[i];
           b->stages[sbase[i] + k] = st;
         }
-        for (size_t k = 0; k < cr.reg_ops.size(); k++) {
-          RegOp r = cr.reg_ops[k];
+        const std::vector<RegOp> lowered = lower_regops(cr);
+        for (size_t k = 0; k < lowered.size(); k++) {
+          RegOp r = lowered[k];
           if (r.mat >= 0) r.mat += pb;
           b->rops[rbase[i] + k] = r;
         }

@@ -673,8 +673,10 @@ static qs_status plan_upload(qs_plan* p, cudaStream_t s) {
   // pageable sources: each copy has read its source when the call returns
   cudaError_t e = cudaSuccess;
   if (p->ops_bytes) e = cudaMemcpyAsync(p->ops_dev, p->cr.tile_ops.data(), p->ops_bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && p->rops_bytes)
-    e = cudaMemcpyAsync(p->rops_dev, p->cr.reg_ops.data(), p->rops_bytes, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && p->rops_bytes) {
+    const std::vector<RegOp> rops = lower_regops(p->cr);
+    e = cudaMemcpyAsync(p->rops_dev, rops.data(), p->rops_bytes, cudaMemcpyHostToDevice, s);
+  }
   if (e == cudaSuccess && p->stages_bytes)
     e = cudaMemcpyAsync(p->stages_dev, p->cr.stages.data(), p->stages_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && p->pool_bytes) e = cudaMemcpyAsync(p->pool_dev, ser.data(), p->pool_bytes, cudaMemcpyHostToDevice, s);

@@ -473,6 +473,54 @@ __device__ __forceinline__ void r_dtab(typename A::reg_t (&x)[1 << K], const typ
   }
 }
 
+// factors on one slot or two (device programs name the slots: no mask test per element)
+template <class A, int K, int S>
+__device__ __forceinline__ void r_neg1(typename A::reg_t (&x)[1 << K]) {
+#pragma unroll
+  for (int j = 0; j < (1 << K); j++)
+    if (j & (1 << S)) x[j] = A::neg(x[j]);
+}
+template <class A, int K, int S>
+__device__ __forceinline__ void r_mul1(typename A::reg_t (&x)[1 << K], const typename A::mat_t& d) {
+#pragma unroll
+  for (int j = 0; j < (1 << K); j++)
+    if (j & (1 << S)) x[j] = A::mul(d, x[j]);
+}
+template <class A, int K, int S0, int S1>
+__device__ __forceinline__ void r_mul2(typename A::reg_t (&x)[1 << K], const typename A::mat_t* m) {
+  const typename A::mat_t d0 = A::ld(m + (1 << S0));
+#pragma unroll
+  for (int j = 0; j < (1 << K); j++)
+    if ((j & (1 << S0)) && !(j & (1 << S1))) x[j] = A::mul(d0, x[j]);
+  const typename A::mat_t d1 = A::ld(m + (1 << S1));
+#pragma unroll
+  for (int j = 0; j < (1 << K); j++)
+    if (!(j & (1 << S0)) && (j & (1 << S1))) x[j] = A::mul(d1, x[j]);
+  const typename A::mat_t d2 = A::ld(m + ((1 << S0) | (1 << S1)));
+#pragma unroll
+  for (int j = 0; j < (1 << K); j++)
+    if ((j & (1 << S0)) && (j & (1 << S1))) x[j] = A::mul(d2, x[j]);
+}
+template <class A, int K, int S0>
+__device__ __forceinline__ void r_mul2_s1(typename A::reg_t (&x)[1 << K], int s1, const typename A::mat_t* m) {
+  if constexpr (K > 1 && S0 < 1) if (s1 == 1) { r_mul2<A, K, S0, (K > 1 ? 1 : 0)>(x, m); return; }
+  if constexpr (K > 2 && S0 < 2) if (s1 == 2) { r_mul2<A, K, S0, (K > 2 ? 2 : 0)>(x, m); return; }
+  if constexpr (K > 3 && S0 < 3) if (s1 == 3) { r_mul2<A, K, S0, (K > 3 ? 3 : 0)>(x, m); return; }
+  if constexpr (K > 4 && S0 < 4) if (s1 == 4) { r_mul2<A, K, S0, (K > 4 ? 4 : 0)>(x, m); return; }
+}
+
+// a phase on the one slot s0, for the groups whose outside controls are set
+template <class A, int K>
+__device__ __forceinline__ void r_phase1(typename A::reg_t (&x)[1 << K], const RegOp& op,
+                                         const typename A::mat_t* __restrict__ m) {
+  if (op.neg) {
+    QS_SLOT_DISPATCH(r_neg1, op.s0, x);
+  } else {
+    const typename A::mat_t d = A::ld(m);
+    QS_SLOT_DISPATCH(r_mul1, op.s0, x, d);
+  }
+}
+
 template <class A, int K>
 __device__ __forceinline__ void apply_regop(typename A::reg_t (&x)[1 << K], const RegOp& op,
                                             const typename A::mat_t* __restrict__ pool, uint32_t gidx,
@@ -517,7 +565,9 @@ __device__ __forceinline__ void apply_regop(typename A::reg_t (&x)[1 << K], cons
     }
     case OP_DTAB: r_dtab<A, K>(x, m, csl); break;
     case OP_PHASE: {
-      if (op.neg) {
+      if (op.s0 >= 0) {
+        r_phase1<A, K>(x, op, m);
+      } else if (op.neg) {
 #pragma unroll
         for (int j = 0; j < (1 << K); j++)
           if ((j & csl) == csl) x[j] = A::neg(x[j]);
@@ -627,18 +677,51 @@ __device__ __forceinline__ void run_reg_stage(typename A::reg_t* T, const StageR
     }
     for (int k = 0; k < sr.nops; k++) {
       const RegOp op = load_regop(rops + sr.op0 + k);
-      if ((base & op.gmask) != op.gmask) continue;
-      // the two most frequent ops (merged tangent-form RX runs and phase tables) skip the
-      // general dispatch; neither carries controls outside the registers
+      // the most frequent ops (merged tangent-form RX runs and phase tables) skip the
+      // general dispatch; they carry no controls outside the registers
       if (op.type == OP_RXTM) {
         r_rxt_multi<A, K>(x, pool + op.mat, op.csl, (uint32_t)(uint8_t)op.neg);
-      } else if (op.type == OP_DTAB) {
+        continue;
+      }
+      if (op.type == OP_DTAB) {
         r_dtab<A, K>(x, pool + op.mat, op.csl);
-      } else if constexpr (Lite) {
-        // passes whose register ops are all of the four kinds below (the host checks): the
+        continue;
+      }
+      if (op.type == OP_DTAB2) {
+        if constexpr (K >= 2) {
+          const typename A::mat_t* m = pool + op.mat;
+          QS_SLOT_DISPATCH(r_mul2_s1, op.s0, x, (int)op.s1, m);
+        }
+        continue;
+      }
+      if constexpr (A::kFrame) {
+        if (op.type == OP_PHASE && op.s1 > 0) {   // a group of phases on one slot: one product
+          const int last = k + op.s1 - 1;
+          typename A::reg_t f;
+          bool any = false;
+          for (; k <= last; k++) {
+            const RegOp o = load_regop(rops + sr.op0 + k);
+            if ((base & o.gmask) != o.gmask || (gidx & o.cot) != o.cot) continue;
+            const typename A::mat_t d = A::ld(pool + o.mat);
+            f = any ? A::mul(d, f) : A::from_mat(d);
+            any = true;
+          }
+          k = last;
+          if (any) {
+            const typename A::mat_t d = A::to_mat(f);
+            QS_SLOT_DISPATCH(r_mul1, op.s0, x, d);
+          }
+          continue;
+        }
+      }
+      if ((base & op.gmask) != op.gmask) continue;
+      if constexpr (Lite) {
+        // passes whose register ops are all of the kinds here (the host checks): the
         // remaining two inline, without the general dispatch's code for the other kinds
         if ((gidx & op.cot) != op.cot) continue;
-        if (op.type == OP_PHASE) {
+        if (op.type == OP_PHASE && op.s0 >= 0) {
+          r_phase1<A, K>(x, op, pool + op.mat);
+        } else if (op.type == OP_PHASE) {
           const uint32_t csl = op.csl;
           if (op.neg) {
 #pragma unroll
@@ -953,6 +1036,43 @@ cudaError_t launch_tile_t(const void* psi, void* dst, const TilePass& tp, const 
 
 }  // namespace
 
+// The instantiations of the policies are compiled side by side: this file is a translation unit of
+// its own (native FP64 and the entry points) and the text of kernels_tile_{f32,df}{,_batched}.cu.
+#define QS_TILE_STAGED(NAME, A)                                                                                     \
+  cudaError_t NAME(const void* psi, void* dst, const TilePass& tp, const StageRec* stages, const RegOp* rops,       \
+                   const DevOp* dops, const void* pool, int* status, cudaStream_t s) {                              \
+    return launch_tile_t<A>(psi, dst, tp, stages, rops, dops, pool, status, s);                                     \
+  }
+#define QS_TILE_BATCHED(NAME, A)                                                                                    \
+  cudaError_t NAME(int K, void* psi, const BatchPass* passes, const uint64_t* prefix, int npass, uint64_t total,    \
+                   int maxL, int minc, const StageRec* stages, const RegOp* rops, const DevOp* dops,                \
+                   const void* pool, int* status, cudaStream_t s) {                                                 \
+    return launch_batched_k<A>(K, psi, passes, prefix, npass, total, maxL, minc, stages, rops, dops, pool, status,  \
+                               s);                                                                                  \
+  }
+#if defined(QS_TILE_F32)
+QS_TILE_STAGED(tile_staged_f32, AF32)
+#elif defined(QS_TILE_F32_BATCHED)
+QS_TILE_BATCHED(tile_batched_f32, AF32)
+#elif defined(QS_TILE_DF)
+QS_TILE_STAGED(tile_staged_df, ADF)
+#elif defined(QS_TILE_DF_BATCHED)
+QS_TILE_BATCHED(tile_batched_df, ADF)
+#else
+QS_TILE_STAGED(tile_staged_f64, AF64)
+QS_TILE_BATCHED(tile_batched_f64, AF64)
+
+#define QS_DECL_STAGED(NAME)                                                                                        \
+  cudaError_t NAME(const void*, void*, const TilePass&, const StageRec*, const RegOp*, const DevOp*, const void*,   \
+                   int*, cudaStream_t)
+#define QS_DECL_BATCHED(NAME)                                                                                       \
+  cudaError_t NAME(int, void*, const BatchPass*, const uint64_t*, int, uint64_t, int, int, const StageRec*,         \
+                   const RegOp*, const DevOp*, const void*, int*, cudaStream_t)
+QS_DECL_STAGED(tile_staged_f32);
+QS_DECL_STAGED(tile_staged_df);
+QS_DECL_BATCHED(tile_batched_f32);
+QS_DECL_BATCHED(tile_batched_df);
+
 int tile_pass_smem_bytes(Policy pol, int L) {
   const int e = (pol == POL_F32) ? 8 : 16;
   return (e << L) + (16 << L) + 16;   // upper bound (padding for c = 0)
@@ -962,9 +1082,9 @@ cudaError_t launch_tile_batched(Policy pol, int K, void* psi, const BatchPass* p
                                 int npass, uint64_t total_blocks, int maxL, int minc, const StageRec* stages,
                                 const RegOp* rops, const DevOp* dops, const void* pool, int* status, cudaStream_t s) {
   switch (pol) {
-    case POL_F32: return launch_batched_k<AF32>(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
-    case POL_F64: return launch_batched_k<AF64>(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
-    case POL_DF: return launch_batched_k<ADF>(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
+    case POL_F32: return tile_batched_f32(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
+    case POL_F64: return tile_batched_f64(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
+    case POL_DF: return tile_batched_df(K, psi, passes, prefix, npass, total_blocks, maxL, minc, stages, rops, dops, pool, status, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -974,11 +1094,13 @@ cudaError_t launch_tile_pass(Policy pol, const void* psi, void* dst, const TileP
                              cudaStream_t s) {
   if (tp.nst == 0 && tp.swap_a == tp.swap_b && psi == dst) return cudaSuccess;
   switch (pol) {
-    case POL_F32: return launch_tile_t<AF32>(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
-    case POL_F64: return launch_tile_t<AF64>(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
-    case POL_DF: return launch_tile_t<ADF>(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
+    case POL_F32: return tile_staged_f32(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
+    case POL_F64: return tile_staged_f64(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
+    case POL_DF: return tile_staged_df(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
   }
   return cudaErrorInvalidValue;
 }
+
+#endif
 
 }  // namespace qs

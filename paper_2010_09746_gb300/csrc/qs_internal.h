@@ -41,6 +41,7 @@ enum OpType : int32_t {
                  // a full-form OP_RX of the same pass
   OP_RXTM = 11,  // register stages only: tangent-form RX on every register slot in csl, in
                  // ascending slot order; pool entries (t, 0) per slot, form bits in neg
+  OP_DTAB2 = 12, // device programs only (lower_regops): a table that depends on slots s0 < s1 alone
 };
 
 struct DevOp {
@@ -291,6 +292,11 @@ int register_bits(int dtype, int L, int requested);
 // Split a pass's op list (tile-local DevOps, program order) into register / shared-memory
 // stages with K register bits; appends to out->stages / reg_ops / tile_ops.
 void build_stages(const std::vector<DevOp>& ops, int L, int K, CompileResult* out, int* st0, int* nst);
+
+// The register ops as the kernels run them (lowering.cpp), one for each of cr.reg_ops and in the same
+// stage ranges: tables and phases on one or two slots get their slots in s0 / s1 (OP_PHASE: s0 >= 0
+// is the only slot of csl, and in double-float plans s1 > 0 counts the phases of its group left).
+std::vector<RegOp> lower_regops(const CompileResult& cr);
 
 // Arithmetic instructions per amplitude of a pass's stages (shared-memory and register ops)
 // as the arithmetic policy's formulas count them: the ALU-work numerator of the roofline.
