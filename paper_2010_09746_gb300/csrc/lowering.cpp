@@ -32,6 +32,11 @@ bool same_entry(const Pool& p, int a, int b) {
 
 // a table whose entries depend on one or two slots only, with entry 1 where neither is set
 void narrow_table(const Pool& pool, int K, RegOp* r) {
+  if (r->csl == 0) {   // every entry is 1: nothing to do (a rotation run without slots)
+    r->type = OP_RXTM;
+    r->neg = 0;
+    return;
+  }
   for (int s = 0; s < K; s++)
     if (r->csl == slot_pattern(s, K)) {
       for (int j = 0; j < (1 << K); j++)
