@@ -32,6 +32,7 @@ struct AF32 {
   using mat_t = float2;
   static constexpr int kStoreBytes = 8;
   static constexpr bool kFrame = false;
+  static constexpr bool kConst = false;
   static __device__ __forceinline__ mat_t ld(const mat_t* p) { return *p; }
   static __device__ __forceinline__ reg_t from_store(store_t v) { return v; }
   static __device__ __forceinline__ store_t to_store(reg_t v) { return v; }
@@ -85,6 +86,7 @@ struct AF64 {
   using mat_t = double2;
   static constexpr int kStoreBytes = 16;
   static constexpr bool kFrame = false;
+  static constexpr bool kConst = false;
   static __device__ __forceinline__ mat_t ld(const mat_t* p) { return *p; }
   static __device__ __forceinline__ reg_t from_store(store_t v) { return v; }
   static __device__ __forceinline__ store_t to_store(reg_t v) { return v; }
@@ -381,6 +383,7 @@ struct ADF {
   using mat_t = dfm;
   static constexpr int kStoreBytes = 16;
   static constexpr bool kFrame = true;
+  static constexpr bool kConst = false;
 
   static QS_HD float2 hi(reg_t v) { return make_float2(v.x, v.y); }
   static QS_HD float2 lo(reg_t v) { return make_float2(v.z, v.w); }
@@ -542,6 +545,17 @@ struct ADF {
     double r = (double)a.x + (double)a.z, i = (double)a.y + (double)a.w;
     return r * r + i * i;
   }
+};
+
+// Policies of the tile kernel whose program sits in the constant bank (kernel parameters): the ops'
+// fields stay uniform, and in ADFC the matrix entries are plain loads, uniform too.
+struct AF32C : AF32 {
+  static constexpr bool kConst = true;
+};
+struct ADFC : ADF {
+  static constexpr bool kConst = true;
+  static __device__ __forceinline__ mat_t ld(const mat_t* p) { return *p; }
+  static __device__ __forceinline__ dfr ld_real(const mat_t* p) { return real_of(*p); }
 };
 
 // one host matrix entry, (re, im) in double, in a policy's format (df_entry: gates.cpp)

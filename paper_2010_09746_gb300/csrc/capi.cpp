@@ -653,10 +653,27 @@ static qs_status plan_upload(qs_plan* p, cudaStream_t s) {
     if (s != p->upload_stream) CUDA_TRY(cudaStreamWaitEvent(s, p->upload_event, 0), "plan upload wait");
     return QS_OK;
   }
-  p->ops_bytes = p->cr.tile_ops.size() * sizeof(DevOp);
-  p->rops_bytes = p->cr.reg_ops.size() * sizeof(RegOp);
-  p->stages_bytes = p->cr.stages.size() * sizeof(StageRec);
-  std::vector<unsigned char> ser = p->cr.pool.serialise(p->pol);
+  int dev = 0, sms = 0;
+  CUDA_TRY(cudaGetDevice(&dev), "device query");
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+  // passes whose program travels with the launch; the device arrays hold what the others need
+  const std::vector<RegOp> rops = lower_regops(p->cr);
+  bool need_arrays = false, need_pool = false;
+  p->progs.assign(p->cr.steps.size(), {});
+  for (size_t i = 0; i < p->cr.steps.size(); i++) {
+    const Step& st = p->cr.steps[i];
+    if (st.kind == ST_PASS && !build_tile_program(p->cr, rops, st.pass, sms, &p->progs[i])) need_arrays = true;
+    if (st.kind == ST_PASS && p->pol == POL_F32) need_pool = true;
+    if (st.kind == ST_GATE && gate_needs_pool(p->pol, st.op)) need_pool = true;
+  }
+  if (need_arrays) {
+    need_pool = true;
+    p->ops_bytes = p->cr.tile_ops.size() * sizeof(DevOp);
+    p->rops_bytes = rops.size() * sizeof(RegOp);
+    p->stages_bytes = p->cr.stages.size() * sizeof(StageRec);
+  }
+  std::vector<unsigned char> ser;
+  if (need_pool) ser = p->cr.pool.serialise(p->pol);
   p->pool_bytes = ser.size();
   p->dense_w_bytes = p->cr.dense_w.size() * sizeof(float);
   if (p->dense_w_bytes) p->dense_w_dev = (float*)dev_alloc(p->dense_w_bytes, s);
@@ -673,10 +690,8 @@ static qs_status plan_upload(qs_plan* p, cudaStream_t s) {
   // pageable sources: each copy has read its source when the call returns
   cudaError_t e = cudaSuccess;
   if (p->ops_bytes) e = cudaMemcpyAsync(p->ops_dev, p->cr.tile_ops.data(), p->ops_bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && p->rops_bytes) {
-    const std::vector<RegOp> rops = lower_regops(p->cr);
+  if (e == cudaSuccess && p->rops_bytes)
     e = cudaMemcpyAsync(p->rops_dev, rops.data(), p->rops_bytes, cudaMemcpyHostToDevice, s);
-  }
   if (e == cudaSuccess && p->stages_bytes)
     e = cudaMemcpyAsync(p->stages_dev, p->cr.stages.data(), p->stages_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && p->pool_bytes) e = cudaMemcpyAsync(p->pool_dev, ser.data(), p->pool_bytes, cudaMemcpyHostToDevice, s);
@@ -689,7 +704,8 @@ static qs_status plan_upload(qs_plan* p, cudaStream_t s) {
 }
 
 static qs_status execute_steps(qs_handle h, qs_plan_t p) {
-  for (const Step& s : p->cr.steps) {
+  for (size_t i = 0; i < p->cr.steps.size(); i++) {
+    const Step& s = p->cr.steps[i];
     const char* name = step_name(s, p->pol);
     if (s.kind == ST_PASS) {
       // a PermuteQubits fused into the pass's store writes the permuted vector to the other
@@ -702,8 +718,9 @@ static qs_status execute_steps(qs_handle h, qs_plan_t p) {
       void* dst = fused ? h->scratch : h->psi;
       CUDA_TRY(timed(h, name, s.bytes,
                      [&] {
+                       const void* prog = p->progs[i].empty() ? nullptr : p->progs[i].data();
                        return launch_tile_pass(p->pol, h->psi, dst, s.pass, p->stages_dev, p->rops_dev, p->ops_dev,
-                                               p->pool_dev, h->status_dev, h->stream);
+                                               p->pool_dev, prog, h->status_dev, h->stream);
                      }, s.alu),
                "tile pass launch");
       if (fused) {

@@ -598,6 +598,13 @@ __device__ __forceinline__ RegOp load_regop(const RegOp* p) {
   return r;
 }
 
+// the same from the constant bank, where the fields stay uniform
+template <class A>
+__device__ __forceinline__ RegOp fetch_op(const RegOp* p) {
+  if constexpr (A::kConst) return *p;
+  else return load_regop(p);
+}
+
 // Phase frame of the double-float policy: while in register format, an element is held as
 // (-i)^popcount(its storage address) times its value, i.e. tile element i of the block at
 // `base` carries (-i)^(popcount(i) + popcount(base)).  Within a pass that is the tile frame times a
@@ -676,7 +683,7 @@ __device__ __forceinline__ void run_reg_stage(typename A::reg_t* T, const StageR
       }
     }
     for (int k = 0; k < sr.nops; k++) {
-      const RegOp op = load_regop(rops + sr.op0 + k);
+      const RegOp op = fetch_op<A>(rops + sr.op0 + k);
       // the most frequent ops (merged tangent-form RX runs and phase tables) skip the
       // general dispatch; they carry no controls outside the registers
       if (op.type == OP_RXTM) {
@@ -700,7 +707,7 @@ __device__ __forceinline__ void run_reg_stage(typename A::reg_t* T, const StageR
           typename A::reg_t f;
           bool any = false;
           for (; k <= last; k++) {
-            const RegOp o = load_regop(rops + sr.op0 + k);
+            const RegOp o = fetch_op<A>(rops + sr.op0 + k);
             if ((base & o.gmask) != o.gmask || (gidx & o.cot) != o.cot) continue;
             const typename A::mat_t d = A::ld(pool + o.mat);
             f = any ? A::mul(d, f) : A::from_mat(d);
@@ -735,6 +742,8 @@ __device__ __forceinline__ void run_reg_stage(typename A::reg_t* T, const StageR
           }
         } else if (op.type == OP_RX) {
           QS_SLOT_DISPATCH(r_rx, op.s0, x, pool + op.mat, op.csl);
+        } else if constexpr (A::kConst) {   // programs in the constant bank may hold these
+          if (op.type == OP_X) QS_SLOT_DISPATCH(r_x, op.s0, x, pool + op.mat, op.csl);
         }
       } else {
         apply_regop<A, K>(x, op, pool, gidx, base);
@@ -835,7 +844,7 @@ __device__ __forceinline__ bool process_block(const typename A::store_t* psi, ty
     if (sr.kind == 0) {
       run_reg_stage<A, K, Lite>(T, sr, rops, pool, L, px, base, in_store, last, df_in, df_out, wb);
       in_store = last;
-    } else {
+    } else if constexpr (!A::kConst) {
       if (kConv && in_store) {
         S* Ts = reinterpret_cast<S*>(T);
         for (uint32_t i = tid; i < nelem; i += kTileThreads) T[px(i)] = load_framed<A>(Ts[px(i)], wb + __popc(i), df_in);
@@ -904,6 +913,25 @@ __global__ void __launch_bounds__(kTileThreads, 2)
   bulk_wait0();
 }
 
+// The pass with its program in the kernel parameters: stages and ops, and with kEntries the matrix
+// entries too (else they are read from pool_dev).
+template <class A, int K, int NB, bool kEntries>
+__global__ void __launch_bounds__(kTileThreads, 2)
+    k_tile_param(const typename A::store_t* psi, typename A::store_t* dst, const __grid_constant__ TileProg<NB> prog,
+                 const typename A::mat_t* __restrict__ pool_dev, int* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const uint32_t bar = init_tile_barrier(smem);
+  const uint64_t nblocks = 1ull << (prog.tp.n - prog.tp.L);
+  const StageRec* stages = reinterpret_cast<const StageRec*>(prog.data);
+  const RegOp* rops = reinterpret_cast<const RegOp*>(prog.data + prog.off_ops);
+  const typename A::mat_t* pool = pool_dev;
+  if constexpr (kEntries) pool = reinterpret_cast<const typename A::mat_t*>(prog.data + prog.off_pool);
+  uint32_t phase = 0;
+  for (uint64_t b = blockIdx.x; b < nblocks; b += gridDim.x)
+    if (!process_block<A, K, true>(psi, dst, prog.tp, b, stages, rops, nullptr, pool, status, smem, bar, phase)) return;
+  bulk_wait0();
+}
+
 // Many independent tile passes in one persistent launch: work item i is block
 // i - prefix[p] of pass p, where prefix[p] <= i < prefix[p + 1]; pass p acts on the state
 // at psi + passes[p].psi_off.
@@ -966,6 +994,27 @@ cudaError_t launch_staged_t(const void* psi, void* dst, const TilePass& tp, cons
   if (grid > nblocks) grid = nblocks;
   k_tile_staged<A, K, Lite><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, tp, stages, rops,
                                                                          dops, (const typename A::mat_t*)pool, status);
+  return cudaGetLastError();
+}
+
+template <class A, int K, int NB, bool kEntries>
+cudaError_t launch_param_t(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t st) {
+  using S = typename A::store_t;
+  const TileProg<NB>& pr = *(const TileProg<NB>*)prog;
+  const TilePass& tp = pr.tp;
+  const size_t smem = kTileSmemOffset + ((size_t)1 << (tp.L - tp.c)) * (((size_t)sizeof(S) << tp.c) + 16);
+  static std::atomic<uint64_t> configured{0};
+  int sms = 0;
+  cudaError_t e = tile_kernel_setup(k_tile_param<A, K, NB, kEntries>, configured, &sms);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_param<A, K, NB, kEntries>, kTileThreads, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const uint64_t nblocks = 1ull << (tp.n - tp.L);
+  uint64_t grid = (uint64_t)sms * per_sm;
+  if (grid > nblocks) grid = nblocks;
+  k_tile_param<A, K, NB, kEntries><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, pr, (const typename A::mat_t*)pool, status);
   return cudaGetLastError();
 }
 
@@ -1037,7 +1086,7 @@ cudaError_t launch_tile_t(const void* psi, void* dst, const TilePass& tp, const 
 }  // namespace
 
 // The instantiations of the policies are compiled side by side: this file is a translation unit of
-// its own (native FP64 and the entry points) and the text of kernels_tile_{f32,df}{,_batched}.cu.
+// its own (native FP64 and the entry points) and the text of kernels_tile_{f32,df}{,_batched}.cu and kernels_tile_param.cu.
 #define QS_TILE_STAGED(NAME, A)                                                                                     \
   cudaError_t NAME(const void* psi, void* dst, const TilePass& tp, const StageRec* stages, const RegOp* rops,       \
                    const DevOp* dops, const void* pool, int* status, cudaStream_t s) {                              \
@@ -1056,6 +1105,13 @@ QS_TILE_STAGED(tile_staged_f32, AF32)
 QS_TILE_BATCHED(tile_batched_f32, AF32)
 #elif defined(QS_TILE_DF)
 QS_TILE_STAGED(tile_staged_df, ADF)
+#elif defined(QS_TILE_PARAM)
+cudaError_t tile_param_f32(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t s) {
+  return launch_param_t<AF32C, 5, kTileProgF32, false>(psi, dst, prog, pool, status, s);
+}
+cudaError_t tile_param_df(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t s) {
+  return launch_param_t<ADFC, 4, kTileProgDF, true>(psi, dst, prog, pool, status, s);
+}
 #elif defined(QS_TILE_DF_BATCHED)
 QS_TILE_BATCHED(tile_batched_df, ADF)
 #else
@@ -1072,6 +1128,8 @@ QS_DECL_STAGED(tile_staged_f32);
 QS_DECL_STAGED(tile_staged_df);
 QS_DECL_BATCHED(tile_batched_f32);
 QS_DECL_BATCHED(tile_batched_df);
+cudaError_t tile_param_f32(const void*, void*, const void*, const void*, int*, cudaStream_t);
+cudaError_t tile_param_df(const void*, void*, const void*, const void*, int*, cudaStream_t);
 
 int tile_pass_smem_bytes(Policy pol, int L) {
   const int e = (pol == POL_F32) ? 8 : 16;
@@ -1090,9 +1148,12 @@ cudaError_t launch_tile_batched(Policy pol, int K, void* psi, const BatchPass* p
 }
 
 cudaError_t launch_tile_pass(Policy pol, const void* psi, void* dst, const TilePass& tp, const StageRec* stages_dev,
-                             const RegOp* regops_dev, const DevOp* ops_dev, const void* pool, int* status_dev,
-                             cudaStream_t s) {
+                             const RegOp* regops_dev, const DevOp* ops_dev, const void* pool, const void* prog,
+                             int* status_dev, cudaStream_t s) {
   if (tp.nst == 0 && tp.swap_a == tp.swap_b && psi == dst) return cudaSuccess;
+  if (prog)
+    return pol == POL_F32 ? tile_param_f32(psi, dst, prog, pool, status_dev, s)
+                          : tile_param_df(psi, dst, prog, pool, status_dev, s);
   switch (pol) {
     case POL_F32: return tile_staged_f32(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);
     case POL_F64: return tile_staged_f64(psi, dst, tp, stages_dev, regops_dev, ops_dev, pool, status_dev, s);

@@ -10,6 +10,8 @@
 // Measured: 25-qubit QFT complex128 (264 controlled phases, in groups of up to 12 on one slot)
 // 9.01 -> 6.17 ms; 23-qubit Haar circuit complex128 16.4 -> 15.9 ms; complex64: 17 qubits
 // 1163 -> 1117 us, 27-qubit RZ/RX/CZ 24.3 -> 23.7 ms, with the same bits.
+#include <string.h>
+
 #include <algorithm>
 
 #include "qs_internal.h"
@@ -98,6 +100,89 @@ std::vector<RegOp> lower_regops(const CompileResult& cr) {
     }
   }
   return ops;
+}
+
+namespace {
+
+// consecutive matrix entries a double-float op reads from its mat on
+int entries_of(const RegOp& r, int K) {
+  switch (r.type) {
+    case OP_DTAB: return 1 << K;
+    case OP_DTAB2: return ((1 << r.s0) | (1 << r.s1)) + 1;
+    case OP_RXTM: return __builtin_popcount(r.csl);
+    case OP_RX: return 2;   // c and s apart
+    case OP_PHASE: return r.neg ? 0 : 1;
+    default: return 0;
+  }
+}
+
+template <int NB>
+bool build_program(const CompileResult& cr, const std::vector<RegOp>& ops, const TilePass& tp,
+                   std::vector<unsigned char>* out) {
+  const bool entries = cr.pol == POL_DF;
+  size_t nops = 0, nent = 0;
+  for (int k = tp.st0; k < tp.st0 + tp.nst; k++) {
+    const StageRec& st = cr.stages[k];
+    if (st.kind != 0) return false;
+    nops += st.nops;
+    for (int i = st.op0; i < st.op0 + st.nops; i++) {
+      const RegOp& r = ops[i];
+      const bool known = r.type == OP_RXTM || r.type == OP_DTAB || r.type == OP_DTAB2 || r.type == OP_PHASE ||
+                         r.type == OP_RX || r.type == OP_X;
+      if (!known) return false;
+      nent += entries ? entries_of(r, tp.K) : 0;
+    }
+  }
+  const size_t off_ops = (tp.nst * sizeof(StageRec) + 15) & ~(size_t)15, off_pool = off_ops + nops * sizeof(RegOp);
+  const size_t eb = Pool::entry_bytes(cr.pol);
+  if (off_pool + nent * eb > (size_t)NB) return false;
+  out->assign(sizeof(TileProg<NB>), 0);
+  TileProg<NB>& p = *(TileProg<NB>*)out->data();
+  p.tp = tp;
+  p.tp.st0 = 0;
+  p.off_ops = (int32_t)off_ops;
+  p.off_pool = (int32_t)off_pool;
+  StageRec* sts = (StageRec*)p.data;
+  RegOp* dst = (RegOp*)(p.data + off_ops);
+  float* pool = (float*)(p.data + off_pool);
+  int o = 0, e = 0;
+  for (int k = 0; k < tp.nst; k++) {
+    sts[k] = cr.stages[tp.st0 + k];
+    const int op0 = sts[k].op0;
+    sts[k].op0 = o;
+    for (int i = op0; i < op0 + sts[k].nops; i++) {
+      RegOp r = ops[i];
+      if (entries) {
+        const int ne = entries_of(r, tp.K);
+        for (int q = 0; q < ne; q++) df_entry(&cr.pool.f64[2 * ((size_t)r.mat + q)], pool + 12 * (e + q));
+        r.mat = e;
+        e += ne;
+      }
+      dst[o++] = r;
+    }
+  }
+  return true;
+}
+
+}  // namespace
+
+// A program in the kernel parameters is used for complex64 at every size and for double-float with no
+// more tiles than SMs (one CTA on an SM).  Constant-bank ops decode in uniform registers, and the
+// kernel holds none of the rarer ops' code.  Measured, device arrays against parameters: complex64
+// Haar circuits of 14 / 17 / 20 / 23 qubits 961 / 1142 / 1518 / 6111 -> 765 / 923 / 1218 / 5298 us, Algorithm 1 at 26
+// qubits 48.6 -> 45.9 ms, the 27-qubit RZ/RX/CZ circuit (passes without moves, which have a light kernel
+// of their own) 24.19 -> 24.28 ms; double-float at 16 / 18 qubits (16 / 64 tiles) 1417 / 1623 -> 1280 / 1457 us, but at
+// 20 qubits (256 tiles) 2076 -> 2246 us and at 23 qubits 15.9 -> 17.0 ms: two CTAs on an SM run through 9 to
+// 30 KB of entries each, past the constant cache.  With ops alone in parameters double-float lost 4 %
+// everywhere, and complex64 entries there lost 8 % at 27 qubits.
+bool build_tile_program(const CompileResult& cr, const std::vector<RegOp>& ops, const TilePass& tp, int sms,
+                        std::vector<unsigned char>* out) {
+  out->clear();
+  if (tp.nst == 0) return false;
+  if (cr.pol == POL_F32 && tp.K == 5) return build_program<kTileProgF32>(cr, ops, tp, out);
+  if (cr.pol == POL_DF && tp.K == 4 && tp.n - tp.L < 31 && (1 << (tp.n - tp.L)) <= sms)
+    return build_program<kTileProgDF>(cr, ops, tp, out);
+  return false;
 }
 
 }  // namespace qs

@@ -104,6 +104,18 @@ struct TilePass {
   int32_t npos[kMaxQubits];          // storage positions of the other bits, ascending
 };
 
+// A tile pass with its program as one kernel parameter: stages at data[0], ops at off_ops and, for
+// double-float, the ops' matrix entries at off_pool (ops index them from 0; complex64 entries stay in
+// the device pool).  The parameter space ends at 32764 bytes.
+template <int NB>
+struct alignas(16) TileProg {
+  TilePass tp;
+  int32_t off_ops, off_pool;
+  alignas(16) unsigned char data[NB];
+};
+constexpr int kTileProgF32 = 16000, kTileProgDF = 32352;
+static_assert(sizeof(TileProg<kTileProgDF>) + 64 <= 32764, "kernel parameter space");
+
 // One pass of a batch: a tile pass on the state that starts psi_off elements into the batch's
 // state buffer.
 struct BatchPass {
@@ -139,11 +151,12 @@ bool gate_needs_pool(Policy pol, const DevOp& op);
 bool block_supported(Policy pol, int k, uint64_t ctl);
 cudaError_t launch_block(Policy pol, void* psi, int n, int k, const int* kq, uint64_t ctl, const double* u,
                          cudaStream_t s);
+// prog: the pass as build_tile_program made it, or NULL (the device arrays are used)
 // reads the state at psi, writes it to dst (the same buffer unless the pass carries a fused
 // permutation, tp.swap_a != tp.swap_b)
 cudaError_t launch_tile_pass(Policy pol, const void* psi, void* dst, const TilePass& tp, const StageRec* stages_dev,
-                             const RegOp* regops_dev, const DevOp* ops_dev, const void* pool, int* status_dev,
-                             cudaStream_t s);
+                             const RegOp* regops_dev, const DevOp* ops_dev, const void* pool, const void* prog,
+                             int* status_dev, cudaStream_t s);
 cudaError_t launch_tile_batched(Policy pol, int K, void* psi, const BatchPass* passes, const uint64_t* prefix,
                                 int npass, uint64_t total_blocks, int maxL, int minc, const StageRec* stages,
                                 const RegOp* rops, const DevOp* dops, const void* pool, int* status, cudaStream_t s);
@@ -297,6 +310,11 @@ void build_stages(const std::vector<DevOp>& ops, int L, int K, CompileResult* ou
 // stage ranges: tables and phases on one or two slots get their slots in s0 / s1 (OP_PHASE: s0 >= 0
 // is the only slot of csl, and in double-float plans s1 > 0 counts the phases of its group left).
 std::vector<RegOp> lower_regops(const CompileResult& cr);
+// The pass (with its lowered ops) as a TileProg in `out`; false (and out empty) where it runs from the
+// device arrays: an op the kernel has no form of, another register width, a program too large for the
+// parameter space, or more double-float tiles than SMs.
+bool build_tile_program(const CompileResult& cr, const std::vector<RegOp>& ops, const TilePass& tp, int sms,
+                        std::vector<unsigned char>* out);
 
 // Arithmetic instructions per amplitude of a pass's stages (shared-memory and register ops)
 // as the arithmetic policy's formulas count them: the ALU-work numerator of the roofline.

@@ -58,6 +58,7 @@ struct qs_plan {
   size_t pool_bytes = 0;
   float* dense_w_dev = nullptr;           // ST_DENSE operands
   size_t dense_w_bytes = 0;
+  std::vector<std::vector<unsigned char>> progs;   // per step: the pass as a kernel parameter, or empty
   bool uploaded = false;
   bool native_alloc = true;
   cudaStream_t upload_stream = nullptr;   // the device copies were enqueued here ...
