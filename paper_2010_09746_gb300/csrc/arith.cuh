@@ -351,12 +351,13 @@ QS_HD double join_double(float hi, float lo) {
 // unnormalised between operations (hi need not be the rounded value of hi + lo);
 // to_store normalises once with TwoSum before the exact integer join.
 //
-// mat_t (48 bytes, prepared on the host) holds a complex u = ur + i ui as lane patterns:
-//   a = ( ur.hi,  ur.hi, -ur.hi, -ur.hi)     ur on both lanes, and its negation
-//   b = (-ui.hi,  ui.hi,  ur.lo,  ur.lo)     (-ui, ui): i ui acting on a swapped (im, re); low part of ur
-//   c = (-ui.lo,  ui.lo, -ur.lo, -ur.lo)     low part of (-ui, ui); negated low part of ur
-// so that u a = ur (.) a + (-ui, ui) (.) swap(a) lane-wise and no packed operand needs a
-// sign flip at run time (a real factor t = ur takes both signs from a, b and c).
+// mat_t (32 bytes, prepared on the host) holds a complex u = ur + i ui as lane patterns:
+//   h = ( ur.hi,  ur.hi, -ui.hi,  ui.hi)     ur on both lanes; (-ui, ui): i ui acting on a swapped (im, re)
+//   l = (-ur.lo, -ur.lo, -ui.lo,  ui.lo)     low parts, that of ur negated
+// so that u a = ur (.) a + (-ui, ui) (.) swap(a) lane-wise; the other sign of ur is two integer
+// operations away.  An entry is read by every lane of a warp, and such a load returns its bytes 32 times
+// over: with both signs stored (48 bytes, three 16-byte loads) the phase tables were bound by
+// those returns (table time at 26 qubits 12.5 ms of 48.4 against 9.6 of arithmetic).
 //
 // Instruction counts per amplitude (packed, two lanes each): u + t v 10, a complex product 14,
 // acc + u a 20.  Each sum of a value and a product is one add_prod2; with a TwoProduct and a
@@ -369,7 +370,7 @@ QS_HD double join_double(float hi, float lo) {
 // (-i)^(popcount r - popcount c)).  The per-gate kernels use the plain frame.
 // ------------------------------------------------------------------------------------------
 struct alignas(16) dfm {
-  float4 a, b, c;
+  float4 h, l;
 };
 // a real double-float factor t as the lane pairs the products need: high and low part on both
 // lanes, and their negations
@@ -390,17 +391,15 @@ struct ADF {
   static QS_HD float2 swp(float2 v) { return make_float2(v.y, v.x); }
   static QS_HD reg_t mk(float2 h, float2 l) { return make_float4(h.x, h.y, l.x, l.y); }
 
-  // A 48-byte entry loaded where it is used: the loads are volatile so that the compiler
-  // cannot hoist the entries of a whole matrix out of a loop (12 registers each).
+  // An entry loaded where it is used: the loads are volatile so that the compiler
+  // cannot hoist the entries of a whole matrix out of a loop (8 registers each).
   static QS_HD mat_t ld(const mat_t* p) {
 #ifdef __CUDA_ARCH__
     mat_t m;
     asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(m.a.x), "=f"(m.a.y), "=f"(m.a.z), "=f"(m.a.w) : "l"(p));
+                 : "=f"(m.h.x), "=f"(m.h.y), "=f"(m.h.z), "=f"(m.h.w) : "l"(p));
     asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4+16];"
-                 : "=f"(m.b.x), "=f"(m.b.y), "=f"(m.b.z), "=f"(m.b.w) : "l"(p));
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4+32];"
-                 : "=f"(m.c.x), "=f"(m.c.y), "=f"(m.c.z), "=f"(m.c.w) : "l"(p));
+                 : "=f"(m.l.x), "=f"(m.l.y), "=f"(m.l.z), "=f"(m.l.w) : "l"(p));
     return m;
 #else
     return *p;
@@ -409,36 +408,30 @@ struct ADF {
   // the real part of an entry (t, 0)
   static QS_HD dfr ld_real(const mat_t* p) {
 #ifdef __CUDA_ARCH__
-    dfr r;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(r.h.x), "=f"(r.h.y), "=f"(r.nh.x), "=f"(r.nh.y) : "l"(p));
-    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+24];" : "=f"(r.l.x), "=f"(r.l.y) : "l"(p));
-    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+40];" : "=f"(r.nl.x), "=f"(r.nl.y) : "l"(p));
-    return r;
+    float2 h, nl;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(h.x), "=f"(h.y) : "l"(p));
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2+16];" : "=f"(nl.x), "=f"(nl.y) : "l"(p));
+    return dfr{h, neg2(h), neg2(nl), nl};
 #else
     return real_of(*p);
 #endif
   }
-  static QS_HD dfr real_of(const mat_t& m) {
-    return dfr{make_float2(m.a.x, m.a.y), make_float2(m.a.z, m.a.w), make_float2(m.b.z, m.b.w),
-               make_float2(m.c.z, m.c.w)};
-  }
+  static QS_HD dfr real_of(const mat_t& m) { return dfr{mA(m), mnA(m), mAl(m), mnAl(m)}; }
   // an entry as an amplitude and back (its own lane patterns of a value that is not normalised)
-  static QS_HD reg_t from_mat(const mat_t& m) { return make_float4(m.a.x, m.b.y, m.b.z, m.c.y); }
+  static QS_HD reg_t from_mat(const mat_t& m) { return make_float4(m.h.x, m.h.w, -m.l.x, m.l.w); }
   static QS_HD mat_t to_mat(reg_t v) {
     mat_t m;
-    m.a = make_float4(v.x, v.x, -v.x, -v.x);
-    m.b = make_float4(-v.y, v.y, v.z, v.z);
-    m.c = make_float4(-v.w, v.w, -v.z, -v.z);
+    m.h = make_float4(v.x, v.x, -v.y, v.y);
+    m.l = make_float4(-v.z, -v.z, -v.w, v.w);
     return m;
   }
   // the lane patterns of an entry
-  static QS_HD float2 mA(const mat_t& m) { return make_float2(m.a.x, m.a.y); }     // ( ur,  ur)
-  static QS_HD float2 mnA(const mat_t& m) { return make_float2(m.a.z, m.a.w); }    // (-ur, -ur)
-  static QS_HD float2 mB(const mat_t& m) { return make_float2(m.b.x, m.b.y); }     // (-ui,  ui)
-  static QS_HD float2 mAl(const mat_t& m) { return make_float2(m.b.z, m.b.w); }    // low parts
-  static QS_HD float2 mnAl(const mat_t& m) { return make_float2(m.c.z, m.c.w); }
-  static QS_HD float2 mBl(const mat_t& m) { return make_float2(m.c.x, m.c.y); }
+  static QS_HD float2 mA(const mat_t& m) { return make_float2(m.h.x, m.h.y); }     // ( ur,  ur)
+  static QS_HD float2 mnA(const mat_t& m) { return neg2(mA(m)); }                  // (-ur, -ur)
+  static QS_HD float2 mB(const mat_t& m) { return make_float2(m.h.z, m.h.w); }     // (-ui,  ui)
+  static QS_HD float2 mnAl(const mat_t& m) { return make_float2(m.l.x, m.l.y); }   // low parts
+  static QS_HD float2 mAl(const mat_t& m) { return neg2(mnAl(m)); }
+  static QS_HD float2 mBl(const mat_t& m) { return make_float2(m.l.z, m.l.w); }
   static QS_HD reg_t from_store(store_t v) {
     const dfl r = split_double(v.x), i = split_double(v.y);
     return make_float4(r.hi, i.hi, r.lo, i.lo);

@@ -128,17 +128,16 @@ HGate make_1q_gate(int q, const cd m[4]) {
   return g;
 }
 
-size_t Pool::entry_bytes(Policy pol) { return pol == POL_F32 ? 8 : (pol == POL_F64 ? 16 : 48); }
+size_t Pool::entry_bytes(Policy pol) { return pol == POL_F32 ? 8 : (pol == POL_F64 ? 16 : 32); }
 
-// double-float lane patterns of u = ur + i ui (12 floats): (ur, ur) and its negation, (-ui, ui)
-// and the low part of (ur, ur), the low part of (-ui, ui) and that of (-ur, -ur)
+// double-float lane patterns of u = ur + i ui (8 floats): (ur, ur), (-ui, ui), and their low parts, that
+// of (ur, ur) negated
 void df_entry(const double* z, float* e) {
   const double ur = z[0], ui = z[1];
   const float rh = (float)ur, rl = (float)(ur - (double)rh);
   const float ih = (float)ui, il = (float)(ui - (double)ih);
-  e[0] = rh; e[1] = rh; e[2] = -rh; e[3] = -rh;
-  e[4] = -ih; e[5] = ih; e[6] = rl; e[7] = rl;
-  e[8] = -il; e[9] = il; e[10] = -rl; e[11] = -rl;
+  e[0] = rh; e[1] = rh; e[2] = -ih; e[3] = ih;
+  e[4] = -rl; e[5] = -rl; e[6] = -il; e[7] = il;
 }
 
 void Pool::serialise_into(Policy pol, unsigned char* dst) const {
@@ -153,7 +152,7 @@ void Pool::serialise_into(Policy pol, unsigned char* dst) const {
     memcpy(dst, f64.data(), E * 16);
   } else {
     float* f = (float*)dst;
-    for (size_t k = 0; k < E; k++) df_entry(&f64[2 * k], f + 12 * k);
+    for (size_t k = 0; k < E; k++) df_entry(&f64[2 * k], f + 8 * k);
   }
 }
 

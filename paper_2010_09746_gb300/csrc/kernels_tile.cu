@@ -466,6 +466,11 @@ __device__ __forceinline__ void r_dtab(typename A::reg_t (&x)[1 << K], const typ
       x[j] = A::mul(M{v.x, v.y}, x[j]);
       x[j + 1] = A::mul(M{v.z, v.w}, x[j + 1]);
     }
+  } else if (__popc(csl) >= (1 << K) - (1 << K) / 8) {
+    // nearly full: without the mask's branches the next entries' loads run ahead of the products, which is
+    // worth more than the one or two products with 1 (exact) that it adds
+#pragma unroll
+    for (int j = 0; j < (1 << K); j++) x[j] = A::mul(A::ld(m + j), x[j]);
   } else {
 #pragma unroll
     for (int j = 0; j < (1 << K); j++)

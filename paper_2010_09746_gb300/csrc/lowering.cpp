@@ -154,7 +154,7 @@ bool build_program(const CompileResult& cr, const std::vector<RegOp>& ops, const
       RegOp r = ops[i];
       if (entries) {
         const int ne = entries_of(r, tp.K);
-        for (int q = 0; q < ne; q++) df_entry(&cr.pool.f64[2 * ((size_t)r.mat + q)], pool + 12 * (e + q));
+        for (int q = 0; q < ne; q++) df_entry(&cr.pool.f64[2 * ((size_t)r.mat + q)], pool + 8 * (e + q));
         r.mat = e;
         e += ne;
       }

@@ -222,7 +222,7 @@ struct FuseOrigin {
   int count(size_t i) const { return off[i + 1] - off[i]; }
 };
 void fuse_single_qubit_runs(int n, std::vector<HGate>& in, bool cz_form, std::vector<HGate>* out, FuseOrigin* origin);
-// one matrix entry, (re, im) in double, as the 12 floats of the double-float lane patterns
+// one matrix entry, (re, im) in double, as the 8 floats of the double-float lane patterns
 void df_entry(const double* z, float* e);
 
 // Matrix pool in policy format.
@@ -234,7 +234,7 @@ struct Pool {
     return (int)(f64.size() / 2 - 1);
   }
   size_t entries() const { return f64.size() / 2; }
-  // serialised for a policy: F32 -> float2, F64 -> double2, DF -> 48-byte lane patterns
+  // serialised for a policy: F32 -> float2, F64 -> double2, DF -> 32-byte lane patterns
   std::vector<unsigned char> serialise(Policy pol) const;
   void serialise_into(Policy pol, unsigned char* dst) const;   // entries() * entry_bytes(pol) bytes
   static size_t entry_bytes(Policy pol);
