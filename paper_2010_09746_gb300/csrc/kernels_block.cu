@@ -8,18 +8,19 @@
 // block of rows at a time and stores every row as it is done: the inputs are in registers, so
 // the update in place needs no second copy of the group.
 //
-// Two ways to bring the amplitudes in, chosen by the lowest target bit (see use_staged):
-//  - direct: thread t's group is group t; for target bits >= 3 (8-byte elements) or >= 2 (16-byte)
-//    the lanes of a warp cover the low bits, and every load and store moves whole sectors;
+// Two ways to bring the amplitudes in, chosen by the low target bits (see use_staged):
+//  - direct: thread t's group is group t; where the lanes of a warp cover the low bits, every load and
+//    store moves whole sectors;
 //  - staged: a warp takes the 2^(K+5) amplitudes over the target bits and the 5 lowest other
 //    bits.  That index set holds the lowest storage bits, so the warp moves them in storage
 //    order, 32 consecutive ranks per instruction, through a padded shared-memory buffer of its
-//    own (no block barrier) from which each lane takes its group.
+//    own (no block barrier) from which each lane takes its group (complex64, two to four qubits).
 //
 // What bounds it: HBM up to K = 4 for complex64 (64 FMA per amplitude against 16 bytes), the FMA
 // pipe at K = 5; double-float arithmetic and the binary64 split / join for complex128.  Measured on
-// a 27-qubit complex64 state: nine blocks (K = 2 .. 5, and one K = 6 on the tensor cores with its
-// permutations) 36.8 -> 5.8 ms; ten 1- and 2-qubit gates on a 26-qubit complex128 state 5.56 -> 4.96 ms.
+// a 27-qubit complex64 state: ten blocks (K = 2 .. 6, low and spread qubits, three of them on the tensor cores)
+// 36.8 -> 5.1 ms, K = 4 on high bits 0.375 ms (5.74 TB/s), K = 5 0.71 ms (24 T FMA/s); complex128 at 26 qubits: K = 1
+// 0.36 ms (5.9 TB/s), K = 2 0.48 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -84,37 +85,62 @@ __device__ __forceinline__ typename A::reg_t block_row(const typename A::mat_t* 
   }
 }
 template <int K>
-struct RowBlock {   // rows computed between two turns of the row loop
+struct RowBlock {   // rows computed between two turns of the row loop (all: more code, nothing gained)
   static constexpr int value = K <= 2 ? (1 << K) : 4;
 };
+// CTAs per SM the registers are limited to: complex64 K = 4 needs the loads of 24 warps in flight
+// (16 warps: 590 us against 375 on a 27-qubit state), K = 5 and complex128 K = 4 hold 64 registers of inputs
+template <class S, int K>
+struct MinCtas {
+  static constexpr int value = K < 4 ? 1 : (K == 4 && sizeof(S) == 8 ? 6 : 4);
+};
 
-template <class A, int K>
-__global__ void __launch_bounds__(kThreads, K >= 4 ? 4 : 1) k_block_direct(typename A::store_t* __restrict__ psi,
-                                                          const __grid_constant__ BlockArgs<K> a,
-                                                          const __grid_constant__ BlockMat<A, K> m) {
+// kPair (complex64): storage bit 0 is target 0 of the block (the launcher orders the targets), so rows r and
+// r + 1 of a group are neighbours and move as 16 bytes
+template <class A, int K, bool kPair>
+__global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::value)
+    k_block_direct(typename A::store_t* __restrict__ psi, const __grid_constant__ BlockArgs<K> a,
+                   const __grid_constant__ BlockMat<A, K> m) {
   using R = typename A::reg_t;
   constexpr int D = 1 << K, RB = RowBlock<K>::value;
   for (uint64_t t = (uint64_t)blockIdx.x * kThreads + threadIdx.x; t < a.nwork; t += (uint64_t)gridDim.x * kThreads) {
     typename A::store_t* p = psi + (expand_bits(t, a.pos, a.nz) | a.ones);
-    typename A::store_t v[D];
     R x[D];
+    if constexpr (kPair) {
+      float4 v[D / 2];
 #pragma unroll
-    for (int r = 0; r < D; r++) v[r] = p[a.off[r]];
+      for (int r = 0; r < D; r += 2) v[r / 2] = *reinterpret_cast<const float4*>(p + a.off[r]);
 #pragma unroll
-    for (int r = 0; r < D; r++) x[r] = A::from_store(v[r]);
+      for (int r = 0; r < D; r += 2) {
+        x[r] = make_float2(v[r / 2].x, v[r / 2].y);
+        x[r + 1] = make_float2(v[r / 2].z, v[r / 2].w);
+      }
+    } else {
+      typename A::store_t v[D];
+#pragma unroll
+      for (int r = 0; r < D; r++) v[r] = p[a.off[r]];
+#pragma unroll
+      for (int r = 0; r < D; r++) x[r] = A::from_store(v[r]);
+    }
 #pragma unroll 1
     for (int r0 = 0; r0 < D; r0 += RB) {
       R y[RB];
 #pragma unroll
       for (int q = 0; q < RB; q++) y[q] = block_row<A, K>(m.u + (r0 + q) * D, x);
+      if constexpr (kPair) {
 #pragma unroll
-      for (int q = 0; q < RB; q++) p[a.off[r0 + q]] = A::to_store(y[q]);
+        for (int q = 0; q < RB; q += 2)
+          *reinterpret_cast<float4*>(p + a.off[r0 + q]) = make_float4(y[q].x, y[q].y, y[q + 1].x, y[q + 1].y);
+      } else {
+#pragma unroll
+        for (int q = 0; q < RB; q++) p[a.off[r0 + q]] = A::to_store(y[q]);
+      }
     }
   }
 }
 
 template <class A, int K>
-__global__ void __launch_bounds__(kThreads, K >= 4 ? 4 : 1) k_block_staged(typename A::store_t* __restrict__ psi,
+__global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::value) k_block_staged(typename A::store_t* __restrict__ psi,
                                                           const __grid_constant__ BlockArgs<K> a,
                                                           const __grid_constant__ BlockMat<A, K> m) {
   using R = typename A::reg_t;
@@ -159,29 +185,49 @@ __global__ void __launch_bounds__(kThreads, K >= 4 ? 4 : 1) k_block_staged(typen
   }
 }
 
-// direct below costs extra sectors and lines per access; staged costs a round trip through shared
-// memory
-template <class S>
-bool use_staged(int lowest_target) {
-  return lowest_target < (sizeof(S) == 16 ? 2 : 3);
+// Which way.  Direct moves 8 or 16 bytes per lane; the sectors and lines that one instruction leaves
+// incomplete are completed by the next ones out of L1 and in L2, which is cheaper than the round trip
+// through shared memory unless the lanes are spread far apart.  27 qubits complex64, us, staged / direct:
+//   K = 2  bits 0 1: 332 / 365   1 2: 331 / 375   0 2: 331 / 336   2 3: 375 / 357   one low bit: 348 / 327
+//   K = 3  bits 0 1 2: 374 / 353   1 2 3: 375 / 503   0 1 and a high one: 379 / 343   one low bit: 402 / 372
+//   K = 4  bits 0-3: 492 / 568   1-4: 492 / 502   2-5: 492 / 373   0 1 and high ones: 495 / 420   one: 501 / 376
+//   K = 5  bits 0-4: 837 / 806   1-5: 839 / 752   one: 849 / 713
+// complex128 (26 qubits): direct 357 against 441 at K = 1 on bit 0, 478 against 522 at K = 2 on bits 0 1, and equal
+// or better beyond.
+bool use_staged(bool c64, int K, uint64_t targets) {
+  if (!c64) return false;
+  if (K == 2) return (targets & ~7ull) == 0;
+  return (K == 3 || K == 4) && (targets & 14ull) == 14ull;
 }
 
 template <class A, int K>
-cudaError_t launch_block_t(void* psi, int n, const int* kq, uint64_t ctl, const double* u, cudaStream_t st) {
+cudaError_t launch_block_t(void* psi, int n, const int* kq_in, uint64_t ctl, const double* u, cudaStream_t st) {
   using S = typename A::store_t;
   constexpr int D = 1 << K;
+  constexpr bool kPairs = std::is_same<A, AF32>::value;
+  // complex64: storage bit 0, where it is a target, becomes target 0 (exchanged with the first one, and the
+  // matrix's rows and columns with it)
+  int kq[K], at0 = -1;
+  for (int b = 0; b < K; b++) {
+    kq[b] = kq_in[b];
+    if (kPairs && kq[b] == 0) at0 = b;
+  }
+  if (at0 > 0) std::swap(kq[0], kq[at0]);
+  auto from = [&](int r) {   // the caller's row or column of ours
+    if (at0 <= 0) return r;
+    const int d = (r ^ (r >> at0)) & 1;
+    return r ^ (d | (d << at0));
+  };
   BlockMat<A, K> m;
-  for (int e = 0; e < D * D; e++) host_entry(u + 2 * e, &m.u[e]);
+  for (int r = 0; r < D; r++)
+    for (int c = 0; c < D; c++) host_entry(u + 2 * (from(r) * D + from(c)), &m.u[r * D + c]);
   BlockArgs<K> a{};
   uint64_t targets = 0;
-  int low = 64;
-  for (int b = 0; b < K; b++) {
-    targets |= 1ull << kq[b];
-    low = std::min(low, kq[b]);
-  }
+  for (int b = 0; b < K; b++) targets |= 1ull << kq[b];
   uint64_t fixed = targets | ctl;
   const int nfree = n - __builtin_popcountll(fixed);
-  const bool staged = use_staged<S>(low) && nfree >= 5;
+  constexpr bool kCanStage = kPairs && K >= 2 && K <= 4;
+  const bool staged = use_staged(kPairs, K, targets) && nfree >= 5;
   a.ones = ctl;
   if (staged) {
     uint64_t lanes = 0, rest = ~fixed;
@@ -227,13 +273,19 @@ cudaError_t launch_block_t(void* psi, int n, const int* kq, uint64_t ctl, const 
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = staged ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_block_staged<A, K>, kThreads, 0)
-               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_block_direct<A, K>, kThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_block_direct<A, K, false>, kThreads, 0);
+  if constexpr (kCanStage)
+    if (e == cudaSuccess && staged) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_block_staged<A, K>, kThreads, 0);
   if (e != cudaSuccess) return e;
   const uint64_t per_block = staged ? kWarps : kThreads;
   const uint64_t grid = std::min<uint64_t>((a.nwork + per_block - 1) / per_block, (uint64_t)sms * std::max(per_sm, 1));
-  if (staged) k_block_staged<A, K><<<(unsigned)grid, kThreads, 0, st>>>((S*)psi, a, m);
-  else k_block_direct<A, K><<<(unsigned)grid, kThreads, 0, st>>>((S*)psi, a, m);
+  if constexpr (kCanStage)
+    if (staged) {
+      k_block_staged<A, K><<<(unsigned)grid, kThreads, 0, st>>>((S*)psi, a, m);
+      return cudaGetLastError();
+    }
+  if (kPairs && at0 >= 0) k_block_direct<A, K, kPairs><<<(unsigned)grid, kThreads, 0, st>>>((S*)psi, a, m);
+  else k_block_direct<A, K, false><<<(unsigned)grid, kThreads, 0, st>>>((S*)psi, a, m);
   return cudaGetLastError();
 }
 
