@@ -360,7 +360,7 @@ QS_HD double join_double(float hi, float lo) {
 // those returns (table time at 26 qubits 12.5 ms of 48.4 against 9.6 of arithmetic).
 //
 // Instruction counts per amplitude (packed, two lanes each): u + t v 10, a complex product 14,
-// acc + u a 20.  Each sum of a value and a product is one add_prod2; with a TwoProduct and a
+// acc + u a 22.  Each sum of a value and a product is one add_prod2; with a TwoProduct and a
 // TwoSum the three took 12, 16 and 24.
 //
 // Tile passes run in a phase frame: amplitude i of a tile is held as (-i)^popcount(i)
@@ -460,18 +460,19 @@ struct ADF {
   static QS_HD reg_t zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
   // U x + V y lane-wise for double-float patterns, U given by its high part and the negated
-  // parts, V by its parts; the two products' low-order terms run in two chains
+  // parts, V by its parts; the two products' low-order terms run in two chains, smallest first
   static QS_HD reg_t dot2(float2 Uh, float2 nUh, float2 nUl, float2 xh, float2 xl, float2 Vh, float2 Vl, float2 yh,
                           float2 yl) {
     const float2 p = mul2(Uh, xh);
     float2 n = fma2(nUh, xh, p);             // -(rounding error of p), exact
-    n = fma2(nUh, xl, n);
     n = fma2(nUl, xh, n);
+    n = fma2(nUh, xl, n);
     float2 s, d, c;
     add_prod2(p, Vh, yh, s, d, c);
-    d = fma2(Vh, yl, d);
+    d = add2(c, d);
     d = fma2(Vl, yh, d);
-    return mk(s, add2(c, sub2(d, n)));
+    d = fma2(Vh, yl, d);
+    return mk(s, sub2(d, n));
   }
   // u a
   static QS_HD reg_t mul(const mat_t& u, reg_t a) {
@@ -483,17 +484,7 @@ struct ADF {
     return mk(s, add2(e, add2(lo(x), lo(y))));
   }
   // acc + u a
-  static QS_HD reg_t mac(reg_t acc, const mat_t& u, reg_t a) {
-    float2 s, d, c, s2, d2, c2;
-    const float2 as = swp(hi(a));
-    add_prod2(hi(acc), mA(u), hi(a), s, d, c);
-    add_prod2(s, mB(u), as, s2, d2, c2);
-    d = fma2(mA(u), lo(a), d);
-    d = fma2(mAl(u), hi(a), d);
-    d2 = fma2(mB(u), swp(lo(a)), d2);
-    d2 = fma2(mBl(u), as, d2);
-    return mk(s2, add2(lo(acc), add2(add2(c, d), add2(c2, d2))));
-  }
+  static QS_HD reg_t mac(reg_t acc, const mat_t& u, reg_t a) { return add(acc, mul(u, a)); }
   // u a + v b
   static QS_HD reg_t mac2(const mat_t& u, reg_t a, const mat_t& v, reg_t b) { return add(mul(u, a), mul(v, b)); }
   // c a - i s b for cs = (c, s), plain frame: c (.) a + (s, -s) (.) swap(b), and (s, -s) is
@@ -507,9 +498,10 @@ struct ADF {
   static QS_HD reg_t add_prod(float2 th, float2 tl, reg_t v, float2 uh, float2 ul) {
     float2 s, d, c;
     add_prod2(uh, th, hi(v), s, d, c);
-    d = fma2(th, lo(v), d);
+    d = add2(c, d);
     d = fma2(tl, hi(v), d);
-    return mk(s, add2(ul, add2(c, d)));
+    d = fma2(th, lo(v), d);
+    return mk(s, add2(ul, d));
   }
   // u + t v
   static QS_HD reg_t axpy_r(const dfr& t, reg_t v, reg_t u) { return add_prod(t.h, t.l, v, hi(u), lo(u)); }
