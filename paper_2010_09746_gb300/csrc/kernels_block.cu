@@ -77,7 +77,7 @@ __device__ __forceinline__ typename A::reg_t block_row(const typename A::mat_t* 
     return A::mac2(u[0], x[0], u[1], x[1]);
   } else {
     typename A::reg_t acc;
-    if constexpr (std::is_same<A, ADF>::value) acc = A::mul(u[0], x[0]);
+    if constexpr (std::is_base_of<ADF, A>::value) acc = A::mul(u[0], x[0]);
     else acc = A::mac(A::zero(), u[0], x[0]);
 #pragma unroll
     for (int c = 1; c < (1 << K); c++) acc = A::mac(acc, u[c], x[c]);
@@ -316,7 +316,7 @@ cudaError_t launch_block(Policy pol, void* psi, int n, int k, const int* kq, uin
   switch (pol) {
     case POL_F32: return launch_block_k<AF32>(psi, n, k, kq, ctl, u, s);
     case POL_F64: return launch_block_k<AF64>(psi, n, k, kq, ctl, u, s);
-    case POL_DF: return launch_block_k<ADF>(psi, n, k, kq, ctl, u, s);
+    case POL_DF: return launch_block_k<ADFG>(psi, n, k, kq, ctl, u, s);
   }
   return cudaErrorInvalidValue;
 }

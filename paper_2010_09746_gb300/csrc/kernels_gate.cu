@@ -514,7 +514,7 @@ cudaError_t launch_gate(Policy pol, void* psi, int n, const DevOp& op, const dou
   switch (pol) {
     case POL_F32: return launch_gate_t<AF32>(pol, psi, n, op, entries, pool, s);
     case POL_F64: return launch_gate_t<AF64>(pol, psi, n, op, entries, pool, s);
-    case POL_DF: return launch_gate_t<ADF>(pol, psi, n, op, entries, pool, s);
+    case POL_DF: return launch_gate_t<ADFG>(pol, psi, n, op, entries, pool, s);
   }
   return cudaErrorInvalidValue;
 }
