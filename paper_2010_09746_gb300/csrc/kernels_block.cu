@@ -16,11 +16,12 @@
 //    order, 32 consecutive ranks per instruction, through a padded shared-memory buffer of its
 //    own (no block barrier) from which each lane takes its group (complex64, two to four qubits).
 //
-// What bounds it: HBM up to K = 4 for complex64 (64 FMA per amplitude against 16 bytes), the FMA
-// pipe at K = 5; double-float arithmetic and the binary64 split / join for complex128.  Measured on
-// a 27-qubit complex64 state: ten blocks (K = 2 .. 6, low and spread qubits, three of them on the tensor cores)
-// 36.8 -> 5.1 ms, K = 4 on high bits 0.375 ms (5.74 TB/s), K = 5 0.71 ms (24 T FMA/s); complex128 at 26 qubits: K = 1
-// 0.36 ms (5.9 TB/s), K = 2 0.48 ms.
+// What bounds it.  complex64: HBM up to K = 4 (64 FMA per amplitude against 16 bytes), the FMA pipe at
+// K = 5.  Double-float: at K = 1, 2 the binary64 split / join and the bytes together, from K = 3 on the FMA
+// pipe (44 * 2^K lane operations per amplitude: 56, 76 and 76 % of it at K = 3, 4, 5).  Measured on a 27-qubit complex64
+// state: ten blocks (K = 2 .. 6, low and spread qubits, three of them on the tensor cores) 36.8 -> 5.0 ms,
+// K = 4 on high bits 0.375 ms (5.74 TB/s), K = 5 0.72 ms (24 T FMA/s); complex128 at 26 qubits: K = 1 0.44 ms
+// (4.8 TB/s), K = 2 0.54, K = 3 0.84, K = 4 1.52, K = 5 3.09 ms (21 ms with one output row per thread).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -50,9 +51,32 @@ struct BlockArgs {
   int lane_rank[5];           // staged: ranks of the lane bits of a group
   int row_pad[1 << K];        // staged: padded position of row r's rank
 };
+// the matrix, row-major
 template <class A, int K>
 struct BlockMat {
   typename A::mat_t u[1 << (2 * K)];
+  __device__ __forceinline__ const typename A::mat_t& at(int i) const { return u[i]; }
+  void set(int i, const double* z) { host_entry(z, &u[i]); }
+};
+// 1024 double-float entries of 32 bytes would be four bytes more than the kernel parameters may take
+// (32764): 24 bytes each, the low parts once and their lane patterns made where they are used
+template <>
+struct BlockMat<ADFG, 5> {
+  float4 h[1024];
+  float2 l[1024];   // (-ur.lo, ui.lo)
+  __device__ __forceinline__ dfm at(int i) const {
+    const float2 v = l[i];
+    dfm m;
+    m.h = h[i];
+    m.l = make_float4(v.x, v.x, -v.y, v.y);
+    return m;
+  }
+  void set(int i, const double* z) {
+    dfm m;
+    host_entry(z, &m);
+    h[i] = m.h;
+    l[i] = make_float2(m.l.x, m.l.w);
+  }
 };
 
 __device__ __forceinline__ uint64_t expand_bits(uint64_t t, const int* pos, int nz) {
@@ -72,37 +96,49 @@ struct PadShift {
 
 // row r of the block on the inputs x
 template <class A, int K>
-__device__ __forceinline__ typename A::reg_t block_row(const typename A::mat_t* u, const typename A::reg_t (&x)[1 << K]) {
+__device__ __forceinline__ typename A::reg_t block_row(const BlockMat<A, K>& m, int r, const typename A::reg_t (&x)[1 << K]) {
+  const int i = r << K;
   if constexpr (K == 1) {
-    return A::mac2(u[0], x[0], u[1], x[1]);
+    return A::mac2(m.at(i), x[0], m.at(i + 1), x[1]);
   } else {
     typename A::reg_t acc;
-    if constexpr (std::is_base_of<ADF, A>::value) acc = A::mul(u[0], x[0]);
-    else acc = A::mac(A::zero(), u[0], x[0]);
+    if constexpr (std::is_base_of<ADF, A>::value) acc = A::mul(m.at(i), x[0]);
+    else acc = A::mac(A::zero(), m.at(i), x[0]);
 #pragma unroll
-    for (int c = 1; c < (1 << K); c++) acc = A::mac(acc, u[c], x[c]);
+    for (int c = 1; c < (1 << K); c++) acc = A::mac(acc, m.at(i + c), x[c]);
     return acc;
   }
 }
-template <int K>
-struct RowBlock {   // rows computed between two turns of the row loop (all: more code, nothing gained)
-  static constexpr int value = K <= 2 ? (1 << K) : 4;
+// How a kernel is compiled.  kRows: rows computed between two turns of the row loop (all: more code,
+// nothing gained).  kCtas: CTAs per SM the registers are limited to.
+//  - complex64 K = 4 needs the loads of 24 warps in flight (16 warps: 590 us against 375 on a 27-qubit
+//    state), K = 5 holds 64 registers of inputs; fewer qubits are at the HBM rate as the compiler leaves them.
+//  - double-float: a thread has long dependent chains before its first load and after its last, so
+//    more warps pay as long as nothing spills.  26 qubits, us, left to the compiler (K = 4: 4 CTAs)
+//    -> limited as here: K = 1 465 -> 444 (8: 470, 12: 472), K = 2 595 -> 540 (10: 549, 12: 566), K = 3
+//    1004 -> 839 (7: 978, 8: 849, 10: 878), K = 4 1870 -> 1521 (3: 1880, 6: 1573).  K = 5 holds 128 registers
+//    of inputs: 3090 at 3 CTAs, 3580 at 2.  Two rows at a time are 2 % better than four at K = 3, four 20 %
+//    worse than two at K = 5.
+//  - native FP64 is bound by its pipe.
+template <class A, int K>
+struct BlockShape {
+  static constexpr int kRows = K <= 2 ? (1 << K) : 4;
+  static constexpr int kCtas = K < 4 ? 1 : (K == 4 && sizeof(typename A::store_t) == 8 ? 6 : 4);
 };
-// CTAs per SM the registers are limited to: complex64 K = 4 needs the loads of 24 warps in flight
-// (16 warps: 590 us against 375 on a 27-qubit state), K = 5 and complex128 K = 4 hold 64 registers of inputs
-template <class S, int K>
-struct MinCtas {
-  static constexpr int value = K < 4 ? 1 : (K == 4 && sizeof(S) == 8 ? 6 : 4);
+template <int K>
+struct BlockShape<ADFG, K> {
+  static constexpr int kRows = K == 2 ? 4 : 2;
+  static constexpr int kCtas = K == 1 ? 16 : K == 2 ? 8 : K == 3 ? 9 : K == 4 ? 5 : 3;
 };
 
 // kPair (complex64): storage bit 0 is target 0 of the block (the launcher orders the targets), so rows r and
 // r + 1 of a group are neighbours and move as 16 bytes
 template <class A, int K, bool kPair>
-__global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::value)
+__global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kCtas)
     k_block_direct(typename A::store_t* __restrict__ psi, const __grid_constant__ BlockArgs<K> a,
                    const __grid_constant__ BlockMat<A, K> m) {
   using R = typename A::reg_t;
-  constexpr int D = 1 << K, RB = RowBlock<K>::value;
+  constexpr int D = 1 << K, RB = BlockShape<A, K>::kRows;
   for (uint64_t t = (uint64_t)blockIdx.x * kThreads + threadIdx.x; t < a.nwork; t += (uint64_t)gridDim.x * kThreads) {
     typename A::store_t* p = psi + (expand_bits(t, a.pos, a.nz) | a.ones);
     R x[D];
@@ -126,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::val
     for (int r0 = 0; r0 < D; r0 += RB) {
       R y[RB];
 #pragma unroll
-      for (int q = 0; q < RB; q++) y[q] = block_row<A, K>(m.u + (r0 + q) * D, x);
+      for (int q = 0; q < RB; q++) y[q] = block_row<A, K>(m, r0 + q, x);
       if constexpr (kPair) {
 #pragma unroll
         for (int q = 0; q < RB; q += 2)
@@ -140,12 +176,12 @@ __global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::val
 }
 
 template <class A, int K>
-__global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::value) k_block_staged(typename A::store_t* __restrict__ psi,
+__global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kCtas) k_block_staged(typename A::store_t* __restrict__ psi,
                                                           const __grid_constant__ BlockArgs<K> a,
                                                           const __grid_constant__ BlockMat<A, K> m) {
   using R = typename A::reg_t;
   using S = typename A::store_t;
-  constexpr int D = 1 << K, RB = RowBlock<K>::value, SH = PadShift<S, K>::value;
+  constexpr int D = 1 << K, RB = BlockShape<A, K>::kRows, SH = PadShift<S, K>::value;
   constexpr int kBuf = (32 << K) + ((32 << K) >> SH);
   __shared__ S bufs[kWarps][kBuf];
   S* buf = bufs[threadIdx.x >> 5];
@@ -176,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, MinCtas<typename A::store_t, K>::val
     for (int r0 = 0; r0 < D; r0 += RB) {
 #pragma unroll
       for (int q = 0; q < RB; q++)
-        buf[lane_pad + a.row_pad[r0 + q]] = A::to_store(block_row<A, K>(m.u + (r0 + q) * D, x));
+        buf[lane_pad + a.row_pad[r0 + q]] = A::to_store(block_row<A, K>(m, r0 + q, x));
     }
     __syncwarp();
 #pragma unroll
@@ -220,7 +256,7 @@ cudaError_t launch_block_t(void* psi, int n, const int* kq_in, uint64_t ctl, con
   };
   BlockMat<A, K> m;
   for (int r = 0; r < D; r++)
-    for (int c = 0; c < D; c++) host_entry(u + 2 * (from(r) * D + from(c)), &m.u[r * D + c]);
+    for (int c = 0; c < D; c++) m.set(r * D + c, u + 2 * (from(r) * D + from(c)));
   BlockArgs<K> a{};
   uint64_t targets = 0;
   for (int b = 0; b < K; b++) targets |= 1ull << kq[b];
@@ -297,7 +333,7 @@ cudaError_t launch_block_k(void* psi, int n, int k, const int* kq, uint64_t ctl,
     case 3: return launch_block_t<A, 3>(psi, n, kq, ctl, u, st);
     case 4: return launch_block_t<A, 4>(psi, n, kq, ctl, u, st);
     case 5:
-      if constexpr (std::is_same<A, AF32>::value) return launch_block_t<A, 5>(psi, n, kq, ctl, u, st);
+      if constexpr (!std::is_same<A, AF64>::value) return launch_block_t<A, 5>(psi, n, kq, ctl, u, st);
       break;
   }
   return cudaErrorInvalidValue;
@@ -305,10 +341,10 @@ cudaError_t launch_block_k(void* psi, int n, int k, const int* kq, uint64_t ctl,
 
 }  // namespace
 
-// Register blocks: up to 32 complex64 or 16 complex128 amplitudes per thread (more would not fit the
-// registers), with at most 6 controls
+// Register blocks: up to 32 amplitudes per thread (16 in native FP64, whose pipe bounds the block at any
+// layout), with at most 6 controls
 bool block_supported(Policy pol, int k, uint64_t ctl) {
-  return k >= 1 && k <= (pol == POL_F32 ? 5 : 4) && __builtin_popcountll(ctl) <= 6;
+  return k >= 1 && k <= (pol == POL_F64 ? 4 : 5) && __builtin_popcountll(ctl) <= 6;
 }
 
 cudaError_t launch_block(Policy pol, void* psi, int n, int k, const int* kq, uint64_t ctl, const double* u,

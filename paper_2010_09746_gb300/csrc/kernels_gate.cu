@@ -186,8 +186,8 @@ __global__ void __launch_bounds__(kThreads) k_diag_c64x2(float2* __restrict__ ps
   }
 }
 
-// dense 2^K x 2^K on bits kq[0..K-1] for the blocks too large for registers (K = 6, and K = 5 of
-// complex128), the matrix in global memory: a block stages kThreads / 2^K groups of 2^K
+// dense 2^K x 2^K on bits kq[0..K-1] for the blocks too large for registers (K = 6, and K = 5 in
+// native FP64), the matrix in global memory: a block stages kThreads / 2^K groups of 2^K
 // amplitudes in shared memory; thread (g, r) computes output row r of group g.
 template <class A, int K>
 __global__ void __launch_bounds__(kThreads) k_dense(typename A::store_t* __restrict__ psi, uint64_t nwork,
@@ -328,7 +328,7 @@ cudaError_t launch_gate_t(Policy pol, void* psi_v, int n, const DevOp& op, const
       const int g = grid_for(nwork << o.nk);
       switch (o.nk) {
         case 5:
-          if constexpr (!std::is_same<A, AF32>::value) k_dense<A, 5><<<g, kThreads, 0, st>>>(psi, nwork, e, o, dm);
+          if constexpr (std::is_same<A, AF64>::value) k_dense<A, 5><<<g, kThreads, 0, st>>>(psi, nwork, e, o, dm);
           break;
         case 6: k_dense<A, 6><<<g, kThreads, 0, st>>>(psi, nwork, e, o, dm); break;
         default: return cudaErrorInvalidValue;
