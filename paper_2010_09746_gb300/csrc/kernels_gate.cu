@@ -60,8 +60,14 @@ struct GateMat {
   typename A::mat_t u[4];
 };
 
+// CTAs per SM the registers of the gate kernels with arithmetic are limited to: double-float hides its
+// chains of conversions and products behind other warps.  26 qubits, us, left to the compiler -> 7
+// CTAs: diag(d0, d1) 473 -> 417 (5: 425), RX 390 -> 379, a phase 213 -> 214.
 template <class A>
-__global__ void __launch_bounds__(kThreads) k_rx(typename A::store_t* __restrict__ psi, uint64_t nwork,
+constexpr int kGateCtas = A::kFrame ? 7 : 1;
+
+template <class A>
+__global__ void __launch_bounds__(kThreads, kGateCtas<A>) k_rx(typename A::store_t* __restrict__ psi, uint64_t nwork,
                                                  Expand e, int p, const __grid_constant__ GateMat<A> m) {
   using R = typename A::reg_t;
   const typename A::mat_t cs = m.u[0];
@@ -77,7 +83,7 @@ __global__ void __launch_bounds__(kThreads) k_rx(typename A::store_t* __restrict
 
 // diag(d0, d1) on bit p, amplitudes with the control bits set
 template <class A>
-__global__ void __launch_bounds__(kThreads) k_diag(typename A::store_t* __restrict__ psi, uint64_t nwork,
+__global__ void __launch_bounds__(kThreads, kGateCtas<A>) k_diag(typename A::store_t* __restrict__ psi, uint64_t nwork,
                                                    Expand e, int p, const __grid_constant__ GateMat<A> m) {
   const typename A::mat_t d0 = m.u[0], d1 = m.u[1];
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
@@ -88,7 +94,7 @@ __global__ void __launch_bounds__(kThreads) k_diag(typename A::store_t* __restri
 
 // multiply by d0 on the amplitudes whose fixed bits (the inserted positions) are all one
 template <class A>
-__global__ void __launch_bounds__(kThreads) k_phase(typename A::store_t* __restrict__ psi, uint64_t nwork,
+__global__ void __launch_bounds__(kThreads, kGateCtas<A>) k_phase(typename A::store_t* __restrict__ psi, uint64_t nwork,
                                                     Expand e, const __grid_constant__ GateMat<A> m) {
   const typename A::mat_t d = m.u[0];
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nwork; t += (uint64_t)gridDim.x * blockDim.x) {
