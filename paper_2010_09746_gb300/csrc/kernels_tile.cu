@@ -903,8 +903,16 @@ __device__ __forceinline__ uint32_t init_tile_barrier(unsigned char* smem) {
   return bar;
 }
 
-template <class A, int K, bool Lite>
-__global__ void __launch_bounds__(kTileThreads, 2)
+// kCtas: CTAs per SM the registers are limited to.  Two (128 registers) where SMs have several tiles, so
+// that one tile's copies run under the other's arithmetic; one (up to 255 registers: no spills, more
+// updates of a stage in flight) for double-float passes with no more tiles than SMs, where a second
+// CTA would have no tile.  Haar / CNOT / CZ circuits of 13 / 16 / 18 qubits: 919 / 1187 / 1352 -> 827 / 1096 /
+// 1242 us, 12 qubits (one tile, programs past the parameter space) 353 -> 339 us.  With more tiles than
+// SMs one CTA of 255 registers loses: 20 / 23 qubits 1.95 / 15.5 -> 2.75 / 18.5 ms, and so do three CTAs of 128 threads
+// (2.57 / 16.7) and two of 192 (2.45 / 18.0), neither of which spills either.  complex64 gains
+// less than 1 % from it.
+template <class A, int K, bool Lite, int kCtas>
+__global__ void __launch_bounds__(kTileThreads, kCtas)
     k_tile_staged(const typename A::store_t* psi, typename A::store_t* dst, const TilePass tp,
                   const StageRec* __restrict__ stages,
                   const RegOp* __restrict__ rops, const DevOp* __restrict__ dops,
@@ -920,8 +928,8 @@ __global__ void __launch_bounds__(kTileThreads, 2)
 
 // The pass with its program in the kernel parameters: stages and ops, and with kEntries the matrix
 // entries too (else they are read from pool_dev).
-template <class A, int K, int NB, bool kEntries>
-__global__ void __launch_bounds__(kTileThreads, 2)
+template <class A, int K, int NB, bool kEntries, int kCtas>
+__global__ void __launch_bounds__(kTileThreads, kCtas)
     k_tile_param(const typename A::store_t* psi, typename A::store_t* dst, const __grid_constant__ TileProg<NB> prog,
                  const typename A::mat_t* __restrict__ pool_dev, int* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -981,28 +989,28 @@ cudaError_t tile_kernel_setup(F* kernel, std::atomic<uint64_t>& configured, int*
   return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
-template <class A, int K, bool Lite>
+template <class A, int K, bool Lite, int kCtas>
 cudaError_t launch_staged_t(const void* psi, void* dst, const TilePass& tp, const StageRec* stages, const RegOp* rops,
                             const DevOp* dops, const void* pool, int* status, cudaStream_t st) {
   using S = typename A::store_t;
   const size_t smem = kTileSmemOffset + ((size_t)1 << (tp.L - tp.c)) * (((size_t)sizeof(S) << tp.c) + 16);
   static std::atomic<uint64_t> configured{0};
   int sms = 0;
-  cudaError_t e = tile_kernel_setup(k_tile_staged<A, K, Lite>, configured, &sms);
+  cudaError_t e = tile_kernel_setup(k_tile_staged<A, K, Lite, kCtas>, configured, &sms);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_staged<A, K, Lite>, kTileThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_staged<A, K, Lite, kCtas>, kTileThreads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const uint64_t nblocks = 1ull << (tp.n - tp.L);
   uint64_t grid = (uint64_t)sms * per_sm;
   if (grid > nblocks) grid = nblocks;
-  k_tile_staged<A, K, Lite><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, tp, stages, rops,
+  k_tile_staged<A, K, Lite, kCtas><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, tp, stages, rops,
                                                                          dops, (const typename A::mat_t*)pool, status);
   return cudaGetLastError();
 }
 
-template <class A, int K, int NB, bool kEntries>
+template <class A, int K, int NB, bool kEntries, int kCtas>
 cudaError_t launch_param_t(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t st) {
   using S = typename A::store_t;
   const TileProg<NB>& pr = *(const TileProg<NB>*)prog;
@@ -1010,16 +1018,16 @@ cudaError_t launch_param_t(const void* psi, void* dst, const void* prog, const v
   const size_t smem = kTileSmemOffset + ((size_t)1 << (tp.L - tp.c)) * (((size_t)sizeof(S) << tp.c) + 16);
   static std::atomic<uint64_t> configured{0};
   int sms = 0;
-  cudaError_t e = tile_kernel_setup(k_tile_param<A, K, NB, kEntries>, configured, &sms);
+  cudaError_t e = tile_kernel_setup(k_tile_param<A, K, NB, kEntries, kCtas>, configured, &sms);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_param<A, K, NB, kEntries>, kTileThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_param<A, K, NB, kEntries, kCtas>, kTileThreads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const uint64_t nblocks = 1ull << (tp.n - tp.L);
   uint64_t grid = (uint64_t)sms * per_sm;
   if (grid > nblocks) grid = nblocks;
-  k_tile_param<A, K, NB, kEntries><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, pr, (const typename A::mat_t*)pool, status);
+  k_tile_param<A, K, NB, kEntries, kCtas><<<(unsigned)grid, kTileThreads, smem, st>>>((const S*)psi, (S*)dst, pr, (const typename A::mat_t*)pool, status);
   return cudaGetLastError();
 }
 
@@ -1029,8 +1037,16 @@ template <class A, int K>
 cudaError_t launch_staged(const void* psi, void* dst, const TilePass& tp, const StageRec* stages, const RegOp* rops,
                           const DevOp* dops, const void* pool, int* status, cudaStream_t st) {
   if constexpr (std::is_same<A, AF32>::value && K == 5)
-    if (tp.flags & kPassLite) return launch_staged_t<A, K, true>(psi, dst, tp, stages, rops, dops, pool, status, st);
-  return launch_staged_t<A, K, false>(psi, dst, tp, stages, rops, dops, pool, status, st);
+    if (tp.flags & kPassLite) return launch_staged_t<A, K, true, 2>(psi, dst, tp, stages, rops, dops, pool, status, st);
+  if constexpr (std::is_same<A, ADF>::value && K == 4) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if ((1ull << (tp.n - tp.L)) <= (uint64_t)sms)
+      return launch_staged_t<A, K, false, 1>(psi, dst, tp, stages, rops, dops, pool, status, st);
+  }
+  return launch_staged_t<A, K, false, 2>(psi, dst, tp, stages, rops, dops, pool, status, st);
 }
 
 template <class A, int K>
@@ -1112,10 +1128,10 @@ QS_TILE_BATCHED(tile_batched_f32, AF32)
 QS_TILE_STAGED(tile_staged_df, ADF)
 #elif defined(QS_TILE_PARAM)
 cudaError_t tile_param_f32(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t s) {
-  return launch_param_t<AF32C, 5, kTileProgF32, false>(psi, dst, prog, pool, status, s);
+  return launch_param_t<AF32C, 5, kTileProgF32, false, 2>(psi, dst, prog, pool, status, s);
 }
 cudaError_t tile_param_df(const void* psi, void* dst, const void* prog, const void* pool, int* status, cudaStream_t s) {
-  return launch_param_t<ADFC, 4, kTileProgDF, true>(psi, dst, prog, pool, status, s);
+  return launch_param_t<ADFC, 4, kTileProgDF, true, 1>(psi, dst, prog, pool, status, s);
 }
 #elif defined(QS_TILE_DF_BATCHED)
 QS_TILE_BATCHED(tile_batched_df, ADF)

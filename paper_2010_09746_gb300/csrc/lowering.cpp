@@ -171,9 +171,10 @@ bool build_program(const CompileResult& cr, const std::vector<RegOp>& ops, const
 // kernel holds none of the rarer ops' code.  Measured, device arrays against parameters: complex64
 // Haar circuits of 14 / 17 / 20 / 23 qubits 961 / 1142 / 1518 / 6111 -> 765 / 923 / 1218 / 5298 us, Algorithm 1 at 26
 // qubits 48.6 -> 45.9 ms, the 27-qubit RZ/RX/CZ circuit (passes without moves, which have a light kernel
-// of their own) 24.19 -> 24.28 ms; double-float at 16 / 18 qubits (16 / 64 tiles) 1417 / 1623 -> 1280 / 1457 us, but at
-// 20 qubits (256 tiles) 2076 -> 2246 us and at 23 qubits 15.9 -> 17.0 ms: two CTAs on an SM run through 9 to
-// 30 KB of entries each, past the constant cache.  With ops alone in parameters double-float lost 4 %
+// of their own) 24.19 -> 24.28 ms; double-float at 16 / 18 qubits (16 / 64 tiles) 1417 / 1623 -> 1280 / 1457 us
+// (1096 / 1242 since the kernel has an SM's registers for one CTA), but at 20 qubits (256 tiles) 2076 -> 2246 us
+// and at 23 qubits 15.9 -> 17.0 ms: two CTAs on an SM run through 9 to 30 KB of entries each, past the
+// constant cache.  With ops alone in parameters double-float lost 4 %
 // everywhere, and complex64 entries there lost 8 % at 27 qubits.
 bool build_tile_program(const CompileResult& cr, const std::vector<RegOp>& ops, const TilePass& tp, int sms,
                         std::vector<unsigned char>* out) {
