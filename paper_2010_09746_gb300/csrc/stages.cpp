@@ -812,18 +812,18 @@ struct Cost {
 };
 double pick(const Cost& c, Policy p) { return p == POL_F32 ? c.f32 : (p == POL_F64 ? c.f64 : c.df); }
 
-const Cost kRX{4, 4, 32};       // two real products and a sum per component
-const Cost kRXT{2, 2, 24};      // one real product and a sum per component (tangent form)
-const Cost kMUL{4, 4, 32};      // complex multiply (diagonal factor, table entry)
-const Cost kU1{8, 8, 80};       // two complex products and a sum
+const Cost kRX{4, 4, 28};       // two real products and a sum per component
+const Cost kRXT{2, 2, 20};      // one real product and a sum per component (tangent form)
+const Cost kMUL{4, 4, 28};      // complex multiply (diagonal factor, table entry)
+const Cost kU1{8, 8, 72};       // two complex products and a sum
 const Cost kNEG{0, 0, 0};       // sign flips
 // amplitude moves (X / CNOT targets, SWAP) do no arithmetic but cost instructions of the
 // same order: register shuffles, and in the double-float phase frame a quarter-turn (lane
 // swap and sign flips) of each moved amplitude.  Counted as instruction equivalents so that
 // circuits made mostly of moves are not predicted free.
 const Cost kMOVE{2, 2, 8};
-const Cost kU2{16, 16, 172};    // per amplitude of a 4x4 block
-const Cost kMACK{4, 4, 46};     // per amplitude per column of a 2^k block
+const Cost kU2{16, 16, 160};    // per amplitude of a 4x4 block
+const Cost kMACK{4, 4, 44};     // per amplitude per column of a 2^k block
 const Cost kCONV{0, 0, 72};     // FP64 <-> (hi, lo) split / join per pass
 
 double fraction(int bits) { return 1.0 / (double)(1u << bits); }
