@@ -290,17 +290,21 @@ void merge_diagonals(std::vector<RegOp>& rl, int K, Pool& pool) {
 // table dropped its entry-0 phase.  Both are scalars on the whole tile, so they commute with
 // every op of the pass and may be applied anywhere in it.  A tangent step multiplies every
 // amplitude by 1 / |dropped factor| (up to sqrt 2), so a pass of hundreds of them would leave
-// the floating-point range; the dropped factors are therefore absorbed in segments: when the
-// current segment's growth would pass 2^seg_bits, the next uncontrolled RX whose cosine is not
-// small (so that no entry leaves 2^-25) keeps the full form and also multiplies by the
-// segment's factors, which brings the magnitudes back.  The
+// the floating-point range; the dropped factors are therefore absorbed in segments: an
+// uncontrolled RX keeps the full form and also multiplies by the segment's factors, which
+// brings the magnitudes back.  A segment is closed by the next RX once its growth would pass
+// 2^soft_bits if that RX's cosine is not small (so that no entry leaves 2^-25), and by any RX
+// once it would pass 2^24: angles near pi drop sines just below 1, and a pass may hold nothing
+// else (a kicked chain of RX(0.85 pi) and CZ).  The
 // last segment's factors and the table phases multiply the first table of the pass (all of
 // its entries then get multiplied), or, in a pass without tables, the pass's first RX, which
-// keeps the full form; magnitudes stay within 2^(+-25) of the unit-norm state.
+// keeps the full form; magnitudes stay within 2^(+-24) of the unit-norm state, and the larger
+// entry of every closing RX is at least 2^-24 / sqrt 2.
 void fold_pass_factors(CompileResult* out, int st0, int nst, int K) {
-  // complex64 closes a segment at any angle, and later: an entry's cosine may be small, which
-  // costs it nothing beside 24-bit products
-  const double seg_bits = out->pol == POL_F32 ? 24.0 : 22.0, min_cos = out->pol == POL_F32 ? 0.0 : 0.25;
+  // complex64 closes a segment at any angle, and as late as it may: an entry's cosine may be
+  // small, which costs it nothing beside 24-bit products
+  constexpr double kHardBits = 24.0, kMinCos = 0.25;
+  const double soft_bits = out->pol == POL_F32 ? kHardBits : 22.0;
   Pool& pool = out->pool;
   const int Dn = 1 << K;   // table entries
   std::vector<int> tabs, rxs;   // indices into out->reg_ops, in execution order
@@ -326,7 +330,7 @@ void fold_pass_factors(CompileResult* out, int st0, int nst, int K) {
     double* e = &pool.f64[2 * (size_t)r.mat];
     const double c = e[0], sn = e[1];
     const double g = -std::log2(std::max(std::fabs(c), std::fabs(sn)));
-    if (grow + g > seg_bits && std::fabs(c) >= min_cos) {   // full form, closing the segment
+    if (grow + g > kHardBits || (grow + g > soft_bits && std::fabs(c) >= kMinCos)) {   // full form, closing the segment
       e[0] *= scale;
       e[1] *= scale;
       scale = 1.0;
