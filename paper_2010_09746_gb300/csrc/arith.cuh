@@ -484,6 +484,12 @@ struct ADF {
     const dfl r = two_sum(v.x, v.z), i = two_sum(v.y, v.w);
     return make_double2(join_double(r.hi, r.lo), join_double(i.hi, i.lo));
   }
+  // the same value with hi the rounded value of hi + lo
+  static QS_HD reg_t normalised(reg_t v) {
+    float2 s, e;
+    two_sum2(hi(v), lo(v), s, e);
+    return mk(s, e);
+  }
   // The double-float storage form a plan keeps between consecutive tile passes: the four
   // floats of a normalised register value in the 16 bytes of an element (no binary64
   // split or join).  It exists only inside one plan execution; the state holds binary64
