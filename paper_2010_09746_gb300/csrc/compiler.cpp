@@ -143,9 +143,12 @@ bool is_identity(const cd m[4]) { return m[0] == cd(1, 0) && m[1] == cd(0, 0) &&
 // gates, or a general one (neither RX nor X in form), or consists of diagonal gates only (one
 // diagonal factor).  A run whose one non-diagonal gate is an RX or an X is kept as it is.
 //
-// A CNOT whose target has such a general run directly before and directly after it is fused
-// as H . CZ . H with the two Hadamards multiplied into those runs, which cost a product
+// A CNOT whose target has a run that is fused to a general matrix directly before and directly after it is
+// fused as H . CZ . H with the two Hadamards multiplied into those runs, which cost a product
 // either way; several CNOTs onto one target with nothing in between share the two Hadamards.
+// On a qubit whose gates so far only move amplitudes and turn their phases (X, Y, S, ...) the CNOT is
+// kept: all of it is exact, as in a circuit of reversible logic, and would not stay so with
+// Hadamards in it.
 // A CZ is diagonal: it needs no qubit in the tile or in registers, so passes and stages hold
 // more gates, and inside a stage it joins the phase tables instead of moving amplitudes
 // (a 23-qubit circuit of 50 layers of Haar gates and CNOT / CZ: 39 -> 35 passes, 138 -> 126
@@ -178,31 +181,35 @@ std::vector<char> cnots_to_cz(int n, const std::vector<HGate>& in) {
   std::vector<char> conv(in.size(), 0);
   struct Q {
     RunShape run;                // since the last multi-qubit gate
+    bool mixed = false;          // a gate on this qubit so far had no zero entry
     std::vector<int> open;       // CNOTs onto this qubit whose run after is not known yet
   };
   std::vector<Q> qs(n);
+  auto fits = [](const Q& s) { return s.mixed && s.run.product(); };
   for (int i = 0; i < (int)in.size(); i++) {
     const HGate& g = in[i];
     if (g.nq == 1) {
-      qs[g.q[0]].run.add(g);
+      Q& s = qs[g.q[0]];
+      s.run.add(g);
+      s.mixed |= g.U[0] != cd(0, 0) && g.U[1] != cd(0, 0);
       continue;
     }
     for (int t = 0; t < g.nq; t++) {
       Q& s = qs[g.q[t]];
       const bool onto = g.kind == QS_OP_CNOT && t == 1;
       if (!s.open.empty() && s.run.size > 0) {   // the sequence ended with this run
-        if (s.run.product())
+        if (fits(s))
           for (int k : s.open) conv[k] = 1;
         s.open.clear();
       } else if (!s.open.empty() && !onto) {     // another gate right after it: no run to fuse into
         s.open.clear();
       }
-      if (onto && (s.run.product() || !s.open.empty())) s.open.push_back(i);
+      if (onto && (fits(s) || !s.open.empty())) s.open.push_back(i);
       s.run = RunShape();
     }
   }
   for (Q& s : qs)
-    if (s.run.product())
+    if (fits(s))
       for (int k : s.open) conv[k] = 1;
   return conv;
 }
