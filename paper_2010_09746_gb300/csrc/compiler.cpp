@@ -130,6 +130,13 @@ void mul2x2(const cd a[4], const cd b[4], cd out[4]) {
   out[3] = r3;
 }
 
+// 1 / sqrt 2 = kRsqrt2 + kRsqrt2Low, the first its nearest double
+constexpr double kRsqrt2 = 0.70710678118654752440, kRsqrt2Low = -4.8336466567264567e-17;
+// a Hadamard, its 1 / sqrt 2 rounded to either side
+bool is_hadamard(const cd m[4]) {
+  return m[0] == m[1] && m[0] == m[2] && m[0] == -m[3] && m[0].imag() == 0.0 &&
+         std::fabs(m[0].real() - kRsqrt2) < 1.2e-16;
+}
 bool is_identity(const cd m[4]) { return m[0] == cd(1, 0) && m[1] == cd(0, 0) && m[2] == cd(0, 0) && m[3] == cd(1, 0); }
 
 }  // namespace
@@ -224,8 +231,7 @@ void fuse_single_qubit_runs(int n, std::vector<HGate>& in, bool cz_form, std::ve
   origin->idx.reserve(in.size());
   // a run's gates in order; kHadamard stands for a Hadamard of a CNOT fused as H . CZ . H
   constexpr int kHadamard = -1;
-  const double rh = std::sqrt(0.5);
-  const cd H[4] = {rh, rh, rh, -rh};
+  const cd sum_diff[4] = {1, 1, 1, -1};   // sqrt 2 times a Hadamard
   std::vector<char> to_cz(in.size(), 0);
   if (cz_form) to_cz = cnots_to_cz(n, in);
   std::vector<std::vector<int>> run(n);
@@ -257,18 +263,24 @@ void fuse_single_qubit_runs(int n, std::vector<HGate>& in, bool cz_form, std::ve
       r.clear();
       return;
     }
+    // In a run with Hadamards of CNOTs every Hadamard, the caller's too, is multiplied in as sums and
+    // differences and the factors 1 / sqrt 2 come last, two of them as an exact 1/2 and an odd one in two
+    // parts: the rounded 1 / sqrt 2 is 7e-17 too large and would scale the state up by as much with
+    // every CNOT.  H next to a CNOT's Hadamard is so the identity to the last bit.
     cd U[4] = {1, 0, 0, 1}, t[4];
-    for (size_t k = 0; k < r.size(); k++) {   // later gates act on the left
-      if (r[k] == kHadamard && k + 1 < r.size() && r[k + 1] == kHadamard) {   // between two CNOTs: H H = 1
-        k++;
-        continue;
-      }
-      cd G[4];
-      for (int e = 0; e < 4; e++) G[e] = r[k] == kHadamard ? H[e] : in[r[k]].U[e];
-      mul2x2(G, U, t);
+    int halves = 0;   // factors 1 / sqrt 2 not multiplied in yet
+    for (int i : r) {   // later gates act on the left
+      const bool h = i == kHadamard || (!all_real && is_hadamard(in[i].U.data()));
+      halves += h;
+      mul2x2(h ? sum_diff : in[i].U.data(), U, t);
       for (int e = 0; e < 4; e++) U[e] = t[e];
     }
-    if (real.empty() && is_identity(U)) {   // two Hadamards that cancelled: no gate is left
+    if (halves) {
+      const double half = std::ldexp(1.0, -(halves / 2)), f = half * kRsqrt2, fl = half * kRsqrt2Low;
+      auto times = [&](double v) { return (halves & 1) ? std::fma(v, f, v * fl) : v * half; };
+      for (int e = 0; e < 4; e++) U[e] = cd(times(U[e].real()), times(U[e].imag()));
+    }
+    if (real.empty() && is_identity(U)) {   // between two CNOTs: H H = 1, no gate is left
       r.clear();
       return;
     }
