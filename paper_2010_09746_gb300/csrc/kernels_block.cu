@@ -113,8 +113,10 @@ __device__ __forceinline__ typename A::reg_t block_row(const BlockMat<A, K>& m, 
 // nothing gained).  kCtas: CTAs per SM the registers are limited to.
 //  - complex64 K = 4 needs the loads of 24 warps in flight (16 warps: 590 us against 375 on a 27-qubit
 //    state), K = 5 holds 64 registers of inputs; fewer qubits are at the HBM rate as the compiler leaves them.
+//    The staged K = 4 kernel would spill 80 bytes at 24 warps: it has a limit of its own, 20 warps
+//    without spills (27 qubits, bits 0-3, us, at 4 / 5 / 6 CTAs: 505 / 465 / 495).
 //  - double-float: a thread has long dependent chains before its first load and after its last, so
-//    more warps pay as long as nothing spills.  26 qubits, us, left to the compiler (K = 4: 4 CTAs)
+//    more warps pay, at K = 3 even with 16 bytes spilled.  26 qubits, us, left to the compiler (K = 4: 4 CTAs)
 //    -> limited as here: K = 1 465 -> 444 (8: 470, 12: 472), K = 2 595 -> 540 (10: 549, 12: 566), K = 3
 //    1004 -> 839 (7: 978, 8: 849, 10: 878), K = 4 1870 -> 1521 (3: 1880, 6: 1573).  K = 5 holds 128 registers
 //    of inputs: 3090 at 3 CTAs, 3580 at 2.  Two rows at a time are 2 % better than four at K = 3, four 20 %
@@ -124,6 +126,7 @@ template <class A, int K>
 struct BlockShape {
   static constexpr int kRows = K <= 2 ? (1 << K) : 4;
   static constexpr int kCtas = K < 4 ? 1 : (K == 4 && sizeof(typename A::store_t) == 8 ? 6 : 4);
+  static constexpr int kStagedCtas = K == 4 ? 5 : kCtas;
 };
 template <int K>
 struct BlockShape<ADFG, K> {
@@ -176,9 +179,9 @@ __global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kCtas)
 }
 
 template <class A, int K>
-__global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kCtas) k_block_staged(typename A::store_t* __restrict__ psi,
-                                                          const __grid_constant__ BlockArgs<K> a,
-                                                          const __grid_constant__ BlockMat<A, K> m) {
+__global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kStagedCtas)
+    k_block_staged(typename A::store_t* __restrict__ psi, const __grid_constant__ BlockArgs<K> a,
+                   const __grid_constant__ BlockMat<A, K> m) {
   using R = typename A::reg_t;
   using S = typename A::store_t;
   constexpr int D = 1 << K, RB = BlockShape<A, K>::kRows, SH = PadShift<S, K>::value;
@@ -226,7 +229,8 @@ __global__ void __launch_bounds__(kThreads, BlockShape<A, K>::kCtas) k_block_sta
 // through shared memory unless the lanes are spread far apart.  27 qubits complex64, us, staged / direct:
 //   K = 2  bits 0 1: 332 / 365   1 2: 331 / 375   0 2: 331 / 336   2 3: 375 / 357   one low bit: 348 / 327
 //   K = 3  bits 0 1 2: 374 / 353   1 2 3: 375 / 503   0 1 and a high one: 379 / 343   one low bit: 402 / 372
-//   K = 4  bits 0-3: 492 / 568   1-4: 492 / 502   2-5: 492 / 373   0 1 and high ones: 495 / 420   one: 501 / 376
+//   K = 4  bits 0-3: 465 / 568   1-4: 465 / 502   2-5: 492 / 373   0 1 and high ones: 495 / 420   one: 501 / 376
+//          (the latter three staged at 24 warps)
 //   K = 5  bits 0-4: 837 / 806   1-5: 839 / 752   one: 849 / 713
 // complex128 (26 qubits): direct 357 against 441 at K = 1 on bit 0, 478 against 522 at K = 2 on bits 0 1, and equal
 // or better beyond.
@@ -305,6 +309,8 @@ cudaError_t launch_block_t(void* psi, int n, const int* kq_in, uint64_t ctl, con
   }
   for (int b = 0; b < n; b++)
     if ((fixed >> b) & 1) a.pos[a.nz++] = b;
+  // The paired form, with fewer registers at K = 2 and 3, takes the plain one's grid too: filled to its own
+  // occupancy it is 3 to 6 % slower with one or two targets low and 5 % faster at K = 3 with bit 0 alone (27 qubits).
   int sms = 0, dev = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
