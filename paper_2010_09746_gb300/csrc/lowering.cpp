@@ -166,12 +166,15 @@ bool build_program(const CompileResult& cr, const std::vector<RegOp>& ops, const
 
 }  // namespace
 
-// A program in the kernel parameters is used for complex64 at every size and for double-float with no
-// more tiles than SMs (one CTA on an SM).  Constant-bank ops decode in uniform registers, and the
-// kernel holds none of the rarer ops' code.  Measured, device arrays against parameters: complex64
-// Haar circuits of 14 / 17 / 20 / 23 qubits 961 / 1142 / 1518 / 6111 -> 765 / 923 / 1218 / 5298 us, Algorithm 1 at 26
-// qubits 48.6 -> 45.9 ms, the 27-qubit RZ/RX/CZ circuit (passes without moves, which have a light kernel
-// of their own) 24.19 -> 24.28 ms; double-float at 16 / 18 qubits (16 / 64 tiles) 1417 / 1623 -> 1280 / 1457 us
+// A program in the kernel parameters is used for complex64, but for passes without moves over many tiles,
+// and for double-float with no more tiles than SMs (one CTA on an SM).  Constant-bank ops decode in uniform
+// registers, and the kernel holds none of the rarer ops' code.  Measured, device arrays against parameters:
+// complex64 Haar circuits of 14 / 17 / 20 / 23 qubits 961 / 1142 / 1518 / 6111 -> 765 / 923 / 1218 / 5298 us, Algorithm 1
+// at 26 qubits 48.6 -> 45.9 ms.  Passes without moves have a light device-array kernel; RZ / RX / CZ circuits of
+// 13 / 18 / 22 / 24 / 26 qubits 169 / 310 / 851 / 3247 / 12216 -> 143 / 267 / 782 / 3157 / 12208 us, but 27 and 28 qubits (2^14 and
+// 2^15 tiles) 24.77 / 31.01 -> 24.89 / 31.25 ms and QFTs of 27 / 29 qubits 11.66 / 50.15 -> 11.84 / 52.12 ms (Algorithm 1 at
+// 27 qubits, whose passes are short, 77.28 -> 77.06): with 50 tiles and more per CTA the program's start no longer counts.
+// Double-float at 16 / 18 qubits (16 / 64 tiles) 1417 / 1623 -> 1280 / 1457 us
 // (1096 / 1242 since the kernel has an SM's registers for one CTA), but at 20 qubits (256 tiles) 2076 -> 2246 us
 // and at 23 qubits 15.9 -> 17.0 ms: two CTAs on an SM run through 9 to 30 KB of entries each, past the
 // constant cache.  With ops alone in parameters double-float lost 4 %
@@ -180,7 +183,8 @@ bool build_tile_program(const CompileResult& cr, const std::vector<RegOp>& ops, 
                         std::vector<unsigned char>* out) {
   out->clear();
   if (tp.nst == 0) return false;
-  if (cr.pol == POL_F32 && tp.K == 5) return build_program<kTileProgF32>(cr, ops, tp, out);
+  const bool light_and_many = (tp.flags & kPassLite) && tp.n - tp.L >= 14;
+  if (cr.pol == POL_F32 && tp.K == 5 && !light_and_many) return build_program<kTileProgF32>(cr, ops, tp, out);
   if (cr.pol == POL_DF && tp.K == 4 && tp.n - tp.L < 31 && (1 << (tp.n - tp.L)) <= sms)
     return build_program<kTileProgDF>(cr, ops, tp, out);
   return false;

@@ -312,7 +312,7 @@ void build_stages(const std::vector<DevOp>& ops, int L, int K, CompileResult* ou
 std::vector<RegOp> lower_regops(const CompileResult& cr);
 // The pass (with its lowered ops) as a TileProg in `out`; false (and out empty) where it runs from the
 // device arrays: an op the kernel has no form of, another register width, a program too large for the
-// parameter space, or more double-float tiles than SMs.
+// parameter space, more double-float tiles than SMs, or a complex64 pass without moves over 2^14 tiles or more.
 bool build_tile_program(const CompileResult& cr, const std::vector<RegOp>& ops, const TilePass& tp, int sms,
                         std::vector<unsigned char>* out);
 
